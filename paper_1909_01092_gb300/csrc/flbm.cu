@@ -205,7 +205,10 @@ int launch_collide(flbm_sim* h, bool fused)
                 h->tm_f[h->cur], h->tm_psi[h->cur], fout, h->st, k, h->tma_wait);                             \
             if (int rc = launch_check(h, "k_collide_bulk_tma")) return rc;                                    \
         } else {                                                                                              \
-            k_collide_bulk<NZ, T1><<<h->grid, h->block, 0, h->stream>>>(fin, fout, psi, h->st, k);            \
+            constexpr unsigned parts = kBulkParts<NZ>;                                                        \
+            k_collide_bulk<NZ, T1><<<dim3(parts * h->grid.x, h->grid.y, h->grid.z),                           \
+                                     dim3(h->block.x, h->block.y / parts), 0, h->stream>>>(fin, fout, psi,     \
+                                                                                           h->st, k);         \
             if (int rc = launch_check(h, "k_collide_bulk")) return rc;                                        \
         }                                                                                                     \
         if (part) CK(h, cudaStreamWaitEvent(h->stream, h->join_ev, 0));                                      \
@@ -283,7 +286,7 @@ int auto_chunk(const KParams& k)
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 148;
     const long long tiles = (long long)k.gx * k.gy;
-    const long long target = 2LL * sms * FLBM_BULK_MINBLOCKS;
+    const long long target = 2LL * sms * kFusedBlocks;
     const long long nch = std::max(1LL, std::min<long long>(k.lz, target / tiles));
     return (int)((k.lz + nch - 1) / nch);
 }

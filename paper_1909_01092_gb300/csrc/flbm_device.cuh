@@ -18,6 +18,8 @@
 #include <cmath>
 #include <cstdint>
 
+#include "flbm_pair.h"
+
 namespace flbm {
 
 // ---------------------------------------------------------------------------
@@ -58,8 +60,7 @@ __host__ __device__ constexpr float bnorm(int k)
 
 // Forward mode transform m_k = sum_i e_k(c_i) f_i of the D3Q19 MRT basis
 // (density, momentum, 6 stress, 9 ghost modes), evaluated with opposite-pair
-// sums (even modes) and differences (odd modes); T = float in the step, double
-// in the observables.
+// sums (even modes) and differences (odd modes); T = double in the observables.
 template <class T>
 __host__ __device__ __forceinline__ void to_modes_t(const T f[19], T m[19])
 {
@@ -98,40 +99,89 @@ __host__ __device__ __forceinline__ void to_modes_t(const T f[19], T m[19])
 
 __host__ __device__ __forceinline__ void to_modes(const float f[19], float m[19]) { to_modes_t<float>(f, m); }
 
-// Back transform f_i = w_i sum_k e_k(c_i) n_k with n_k = m_k / b_k already
-// normalised, split into the even and odd parts of each opposite pair.
-__host__ __device__ __forceinline__ void from_modes(const float n[19], float f[19])
+// The same transform in packed arithmetic (both components at once), every
+// operation written out.
+__device__ __forceinline__ void to_modes(const Pair f[19], Pair m[19])
 {
-    const float k18 = 1.0f / 18.0f, k36 = 1.0f / 36.0f;
-    f[0] = (n[0] - n[4] + n[16]) * (1.0f / 3.0f);
-    const float ex = (n[0] + 2.0f * n[5] - 2.0f * n[16] - 2.0f * n[17]) * k18;
-    const float ox = (n[1] - 2.0f * n[10]) * k18;
-    const float ey = (n[0] - n[5] + n[6] - 2.0f * n[16] + n[17] - n[18]) * k18;
-    const float oy = (n[2] - 2.0f * n[11]) * k18;
-    const float ez = (n[0] - n[5] - n[6] - 2.0f * n[16] + n[17] + n[18]) * k18;
-    const float oz = (n[3] - 2.0f * n[12]) * k18;
-    const float cmn = n[0] + n[4] + n[16];
-    const float exy = cmn + n[5] + n[6] + n[17] + n[18];
-    const float exz = cmn + n[5] - n[6] + n[17] - n[18];
-    const float eyz = cmn - 2.0f * n[5] - 2.0f * n[17];
-    const float e7 = (exy + n[7]) * k36, e9 = (exy - n[7]) * k36;
-    const float o7 = (n[1] + n[2] + n[10] + n[11] + n[13] - n[14]) * k36;
-    const float o9 = (n[1] - n[2] + n[10] - n[11] + n[13] + n[14]) * k36;
-    const float e11 = (exz + n[9]) * k36, e13 = (exz - n[9]) * k36;
-    const float o11 = (n[1] + n[3] + n[10] + n[12] - n[13] + n[15]) * k36;
-    const float o13 = (n[1] - n[3] + n[10] - n[12] - n[13] - n[15]) * k36;
-    const float e15 = (eyz + n[8]) * k36, e17 = (eyz - n[8]) * k36;
-    const float o15 = (n[2] + n[3] + n[11] + n[12] + n[14] - n[15]) * k36;
-    const float o17 = (n[2] - n[3] + n[11] - n[12] + n[14] + n[15]) * k36;
-    f[1] = ex + ox; f[2] = ex - ox;
-    f[3] = ey + oy; f[4] = ey - oy;
-    f[5] = ez + oz; f[6] = ez - oz;
-    f[7] = e7 + o7; f[8] = e7 - o7;
-    f[9] = e9 + o9; f[10] = e9 - o9;
-    f[11] = e11 + o11; f[12] = e11 - o11;
-    f[13] = e13 + o13; f[14] = e13 - o13;
-    f[15] = e15 + o15; f[16] = e15 - o15;
-    f[17] = e17 + o17; f[18] = e17 - o17;
+    const Pair two = splat(2.0f), mtwo = splat(-2.0f);
+    const Pair s1 = add(f[1], f[2]), d1 = sub(f[1], f[2]);
+    const Pair s2 = add(f[3], f[4]), d2 = sub(f[3], f[4]);
+    const Pair s3 = add(f[5], f[6]), d3 = sub(f[5], f[6]);
+    const Pair s7 = add(f[7], f[8]), d7 = sub(f[7], f[8]);
+    const Pair s9 = add(f[9], f[10]), d9 = sub(f[9], f[10]);
+    const Pair s11 = add(f[11], f[12]), d11 = sub(f[11], f[12]);
+    const Pair s13 = add(f[13], f[14]), d13 = sub(f[13], f[14]);
+    const Pair s15 = add(f[15], f[16]), d15 = sub(f[15], f[16]);
+    const Pair s17 = add(f[17], f[18]), d17 = sub(f[17], f[18]);
+    const Pair s23 = add(s2, s3), sax = add(s1, s23);
+    const Pair sxy = add(s7, s9), sxz = add(s11, s13), syz = add(s15, s17);
+    const Pair sxx = add(sxy, sxz), sdg = add(sxx, syz);
+    // the odd sums of the diagonal directions, per axis
+    const Pair ax = add(add(d7, d9), add(d11, d13));
+    const Pair ay = add(sub(d7, d9), add(d15, d17));
+    const Pair az = add(sub(d11, d13), sub(d15, d17));
+    m[0] = add(f[0], add(sax, sdg));
+    m[1] = add(d1, ax);
+    m[2] = add(d2, ay);
+    m[3] = add(d3, az);
+    m[4] = sub(sdg, f[0]);
+    const Pair sq = mad(mtwo, syz, sxx);  // s_xy + s_xz - 2 s_yz
+    const Pair sr = mad(two, s1, mul(splat(-1.0f), s23));
+    m[5] = add(sr, sq);
+    const Pair d23 = sub(s2, s3), dxx = sub(sxy, sxz);
+    m[6] = add(d23, dxx);
+    m[7] = sub(s7, s9);
+    m[8] = sub(s15, s17);
+    m[9] = sub(s11, s13);
+    m[10] = mad(mtwo, d1, ax);
+    m[11] = mad(mtwo, d2, ay);
+    m[12] = mad(mtwo, d3, az);
+    m[13] = sub(add(d7, d9), add(d11, d13));
+    m[14] = sub(add(d15, d17), sub(d7, d9));
+    m[15] = sub(sub(d11, d13), sub(d15, d17));
+    m[16] = add(f[0], mad(mtwo, sax, sdg));
+    m[17] = sub(sq, sr);
+    m[18] = sub(dxx, d23);
+}
+
+// Back transform f_i = w_i sum_k e_k(c_i) n_k with n_k = m_k / b_k already
+// normalised, split into the even and odd parts of each opposite pair; T =
+// Pair in the step (both components at once).
+template <class T>
+__host__ __device__ __forceinline__ void from_modes(const T n[19], T f[19])
+{
+    const T two = lit<T>(2.0f), mtwo = lit<T>(-2.0f);
+    const T k18 = lit<T>(1.0f / 18.0f), k36 = lit<T>(1.0f / 36.0f);
+    const T m18 = lit<T>(-1.0f / 18.0f), m36 = lit<T>(-1.0f / 36.0f);
+    f[0] = mul(add(sub(n[0], n[4]), n[16]), lit<T>(1.0f / 3.0f));
+    const T a = mad(mtwo, n[16], n[0]);
+    const T p = sub(n[5], n[17]), q = sub(n[6], n[18]);
+    const T ap = sub(a, p);
+    const T ex = mul(mad(two, p, a), k18), ey = mul(add(ap, q), k18), ez = mul(sub(ap, q), k18);
+    const T ox = mad(mtwo, n[10], n[1]), oy = mad(mtwo, n[11], n[2]), oz = mad(mtwo, n[12], n[3]);
+    f[1] = mad(ox, k18, ex); f[2] = mad(ox, m18, ex);
+    f[3] = mad(oy, k18, ey); f[4] = mad(oy, m18, ey);
+    f[5] = mad(oz, k18, ez); f[6] = mad(oz, m18, ez);
+    const T cmn = add(add(n[0], n[4]), n[16]);
+    const T s = add(n[5], n[17]), t = add(n[6], n[18]);
+    const T cs = add(cmn, s);
+    const T exy = add(cs, t), exz = sub(cs, t), eyz = mad(mtwo, s, cmn);
+    const T e7 = mul(add(exy, n[7]), k36), e9 = mul(sub(exy, n[7]), k36);
+    const T e11 = mul(add(exz, n[9]), k36), e13 = mul(sub(exz, n[9]), k36);
+    const T e15 = mul(add(eyz, n[8]), k36), e17 = mul(sub(eyz, n[8]), k36);
+    const T X = add(n[1], n[10]), Y = add(n[2], n[11]), Z = add(n[3], n[12]);
+    const T x7 = add(X, n[13]), y7 = sub(Y, n[14]);
+    const T x11 = sub(X, n[13]), z11 = add(Z, n[15]);
+    const T y15 = add(Y, n[14]), z15 = sub(Z, n[15]);
+    const T o7 = add(x7, y7), o9 = sub(x7, y7);
+    const T o11 = add(x11, z11), o13 = sub(x11, z11);
+    const T o15 = add(y15, z15), o17 = sub(y15, z15);
+    f[7] = mad(o7, k36, e7); f[8] = mad(o7, m36, e7);
+    f[9] = mad(o9, k36, e9); f[10] = mad(o9, m36, e9);
+    f[11] = mad(o11, k36, e11); f[12] = mad(o11, m36, e11);
+    f[13] = mad(o13, k36, e13); f[14] = mad(o13, m36, e13);
+    f[15] = mad(o15, k36, e15); f[16] = mad(o15, m36, e15);
+    f[17] = mad(o17, k36, e17); f[18] = mad(o17, m36, e17);
 }
 
 // ---------------------------------------------------------------------------

@@ -113,8 +113,10 @@ static __global__ void __launch_bounds__(256) kb_shell(const RepDesc* __restrict
     FLBM_END_ITEMS
 }
 
+// Two blocks per SM: the descriptor read from shared memory leaves the update
+// 216 bytes of spills at three.
 template <bool NOISE, bool TAU1>
-static __global__ void __launch_bounds__(256, 3)
+static __global__ void __launch_bounds__(256, 2)
     kb_bulk(const RepDesc* __restrict__ reps, const Item* __restrict__ items, int nitems, int par)
 {
     FLBM_FOR_ITEMS
@@ -136,23 +138,26 @@ struct RepChunk {
 static_assert(sizeof(RepChunk) + 64 <= 32764, "kernel parameters are at most 32764 bytes");
 
 template <bool NOISE, bool TAU1>
-static __global__ void __launch_bounds__(256, 4) kb_bulk_rep(const __grid_constant__ RepChunk c, int par)
+static __global__ void __launch_bounds__(kBulkThreads<NOISE>, kBulkBlocks<NOISE>)
+    kb_bulk_rep(const __grid_constant__ RepChunk c, int par)
 {
+    constexpr int parts = kBulkParts<NOISE>;
     const RepDesc& R = c.r[blockIdx.y];
     const KParams& P = R.P;
     const int plane = P.gx * P.gy;
-    const int t = blockIdx.x;
+    const int t = blockIdx.x / parts;
     if (t >= plane * P.lz) return;
     const int bz = t / plane, w = t - bz * plane;
     const int by = w / P.gx, bx = w - by * P.gx;
-    const int tx = threadIdx.x & (P.tx - 1), ty = threadIdx.x >> (__ffs(P.tx) - 1);
+    const int tid = threadIdx.x + kBulkThreads<NOISE> * (blockIdx.x % parts);
+    const int tx = tid & (P.tx - 1), ty = tid >> (__ffs(P.tx) - 1);
     bulk_tile<NOISE, TAU1>(bx, by, bz, tx, ty, R.f[par], R.f[1 - par], R.psi, R.st, P);
 }
 
-// Three blocks per SM: the register cap costs some spills, and the extra
-// resident warps hide more of the near tiles' latency (measured faster).
+// Two blocks per SM, without spills (step of the confinement channels, where
+// most tiles are near: 1.13 ms against 1.32 ms at three, bulk lists included).
 template <bool NOISE, bool TAU1>
-static __global__ void __launch_bounds__(256, 3)
+static __global__ void __launch_bounds__(256, 2)
     kb_near(const RepDesc* __restrict__ reps, const Item* __restrict__ items, int nitems, int par)
 {
     FLBM_FOR_ITEMS
@@ -476,7 +481,9 @@ int launch_bulk_reps(flbm_ens* e, int par)
                                             kb_bulk_rep<true, false>, kb_bulk_rep<true, true>};
     for (int k = 0; k < 4; ++k)
         for (const auto& ch : e->rep_launches[k]) {
-            kern[k]<<<dim3((unsigned)ch.max_blocks, (unsigned)ch.n), 256, 0, e->stream>>>(ch.c, par);
+            const unsigned parts = k >= 2 ? kBulkParts<true> : kBulkParts<false>;
+            const unsigned threads = k >= 2 ? kBulkThreads<true> : kBulkThreads<false>;
+            kern[k]<<<dim3(parts * (unsigned)ch.max_blocks, (unsigned)ch.n), threads, 0, e->stream>>>(ch.c, par);
             if (int rc = elaunch(e, "kb_bulk_rep")) return rc;
         }
     return FLBM_OK;

@@ -314,8 +314,10 @@ struct RingDuty {
     }
 };
 
+constexpr int kFusedBlocks = 4;  // resident blocks per SM of the fused collide
+
 template <bool NOISE, bool TAU1>
-static __global__ void __launch_bounds__(kThreadsStep, FLBM_BULK_MINBLOCKS)
+static __global__ void __launch_bounds__(kThreadsStep, kFusedBlocks)
     k_collide_bulk_fused(const float* __restrict__ fin, float* __restrict__ fout, const float* __restrict__ psi,
                          float* __restrict__ psi_next, float2* __restrict__ ring, float2* __restrict__ seam,
                          const DevState* __restrict__ st, KParams P, FusedGeom G)

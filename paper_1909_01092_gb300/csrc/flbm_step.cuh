@@ -18,10 +18,6 @@
 
 #include "flbm_device.cuh"
 
-#ifndef FLBM_BULK_MINBLOCKS
-#define FLBM_BULK_MINBLOCKS 4  // resident 256-thread blocks per SM the bulk kernel is compiled for
-#endif
-
 namespace flbm {
 
 // Philox4x32-10 with the round keys precomputed on the host (key + r * Weyl).
@@ -43,30 +39,65 @@ __host__ __device__ __forceinline__ void philox_rk(uint32_t& x0, uint32_t& x1, u
     }
 }
 
-// Box-Muller pair from two Philox words with the hardware approximations of
-// log2, rsqrt, sin and cos: z0 = r cos(2 pi u2), z1 = r sin(2 pi u2) with
-// r = sqrt(-2 ln u1); the angle is taken as 2 pi (u2 - 1/2) in (-pi, pi),
-// where the approximations are accurate, and the signs flipped back. The
-// flush-to-zero forms are used: their inputs and results here (u1 >= 2^-24,
-// |angle| >= 2^-22, -2 ln u1 of about 2^-23 at least) lie far above the
-// subnormal range, where both forms agree, and they skip the rescaling of
-// subnormal inputs.
-__device__ __forceinline__ void box_muller(uint32_t w1, uint32_t w2, float& z0, float& z1)
+// Two Box-Muller pairs from four Philox words (w1, w2 -> za0, za1; w3, w4 ->
+// zb0, zb1) with the hardware approximations of log2, rsqrt, sin and cos:
+// z0 = r cos(2 pi u2), z1 = r sin(2 pi u2) with r = sqrt(-2 ln u1); the angle
+// is taken as 2 pi (u2 - 1/2) in (-pi, pi), where the approximations are
+// accurate, and the signs flipped back. The flush-to-zero forms are used:
+// their inputs and results here (u1 >= 2^-24, |angle| >= 2^-22, -2 ln u1 of
+// about 2^-23 at least) lie far above the subnormal range, where both forms
+// agree, and they skip the rescaling of subnormal inputs.
+// A word's upper 23 bits become the fraction of a float in [1, 2) by one
+// funnel shift (0x7f above the word puts the exponent of 1 in front), so the
+// uniforms need no integer conversion, which shares the slow pipe of the four
+// approximations: u = ((w >> 9) + 1/2) 2^-23 = float - (1 - 2^-24), exact.
+// The rest of the arithmetic is packed over the two pairs.
+__device__ __forceinline__ Pair one_to_two(uint32_t w1, uint32_t w3)
 {
-    const float u1 = uniform_open(w1);
-    float lg, rs, s, c;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(u1));
-    const float e = -1.38629436112f * lg;  // -2 ln u1 > 0
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(e));
-    const float r = e * rs;
-    // 2 pi (u2 - 1/2) with u2 = ((w2 >> 9) + 1/2) 2^-23, as one multiply-add.
-    constexpr float kA = (float)(6.283185307179586 / 8388608.0);
+    return Pair{__uint_as_float(__funnelshift_r(w1, 0x7fu, 9)), __uint_as_float(__funnelshift_r(w3, 0x7fu, 9))};
+}
+
+__device__ __forceinline__ void box_muller2(uint32_t w1, uint32_t w2, uint32_t w3, uint32_t w4, float& za0, float& za1,
+                                            float& zb0, float& zb1)
+{
+    const Pair u1 = add(one_to_two(w1, w3), splat(-0.999999940395355224609375f));
+    Pair lg, rs, s, c;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg.x) : "f"(u1.x));
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg.y) : "f"(u1.y));
+    const Pair e = mul(lg, splat(-1.38629436112f));  // -2 ln u1 > 0
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs.x) : "f"(e.x));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs.y) : "f"(e.y));
+    const Pair r = mul(e, rs);
+    // 2 pi (u2 - 1/2) with u2 = ((w2 >> 9) + 1/2) 2^-23.
+    constexpr float kA = (float)6.283185307179586;
     constexpr float kB = (float)(6.283185307179586 * (0.5 / 8388608.0 - 0.5));
-    const float ang = __fmaf_rn((float)(w2 >> 9), kA, kB);
-    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(ang));
-    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(ang));
-    z0 = -r * c;
-    z1 = -r * s;
+    const Pair ang = mad(add(one_to_two(w2, w4), splat(-1.0f)), splat(kA), splat(kB));
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(s.x) : "f"(ang.x));
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(c.x) : "f"(ang.x));
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(s.y) : "f"(ang.y));
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(c.y) : "f"(ang.y));
+    za0 = -r.x * c.x;
+    za1 = -r.x * s.x;
+    zb0 = -r.y * c.y;
+    zb1 = -r.y * s.y;
+}
+
+// 1 / x and sqrt(x) for finite x > 0 (sqrt: x >= 0) from the hardware's
+// approximations and one Newton step each, to within an ulp, without the
+// branches and calls of the general routines. Zero gives 0 for the square
+// root; a NaN stays one.
+__device__ __forceinline__ float recip_newton(float x)
+{
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return __fmaf_rn(r, __fmaf_rn(-x, r, 1.0f), r);
+}
+__device__ __forceinline__ float sqrt_newton(float x)
+{
+    float y;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(x, 1.17549435e-38f)));
+    const float s = __fmul_rn(x, y);
+    return __fmaf_rn(__fmaf_rn(-s, s, x), __fmul_rn(0.5f, y), s);
 }
 
 // FP32 sums over the particle links of one node.
@@ -86,38 +117,61 @@ __device__ __forceinline__ void link_add(LinkSums& s, float m, int cx, int cy, i
     s.T[2] += 0.5f * (cx * fr[1] - cy * fr[0]);
 }
 
-// Density and momentum of one component from its 19 populations.
-__device__ __forceinline__ void moments(const float f[19], float& rho, float j[3])
+// Densities and momenta of both components from their populations.
+__device__ __forceinline__ void moments(const Pair f[19], Pair& rho, Pair j[3])
 {
-    const float s1 = f[1] + f[2], s2 = f[3] + f[4], s3 = f[5] + f[6];
-    const float s7 = f[7] + f[8], s9 = f[9] + f[10], s11 = f[11] + f[12];
-    const float s13 = f[13] + f[14], s15 = f[15] + f[16], s17 = f[17] + f[18];
-    const float d7 = f[7] - f[8], d9 = f[9] - f[10], d11 = f[11] - f[12];
-    const float d13 = f[13] - f[14], d15 = f[15] - f[16], d17 = f[17] - f[18];
-    rho = f[0] + (s1 + s2 + s3) + (s7 + s9) + (s11 + s13) + (s15 + s17);
-    j[0] = (f[1] - f[2]) + d7 + d9 + d11 + d13;
-    j[1] = (f[3] - f[4]) + d7 - d9 + d15 + d17;
-    j[2] = (f[5] - f[6]) + d11 - d13 + d15 - d17;
+    const Pair s1 = add(f[1], f[2]), s2 = add(f[3], f[4]), s3 = add(f[5], f[6]);
+    const Pair s7 = add(f[7], f[8]), s9 = add(f[9], f[10]), s11 = add(f[11], f[12]);
+    const Pair s13 = add(f[13], f[14]), s15 = add(f[15], f[16]), s17 = add(f[17], f[18]);
+    const Pair d7 = sub(f[7], f[8]), d9 = sub(f[9], f[10]), d11 = sub(f[11], f[12]);
+    const Pair d13 = sub(f[13], f[14]), d15 = sub(f[15], f[16]), d17 = sub(f[17], f[18]);
+    const Pair sax = add(add(s1, s2), s3);
+    const Pair sdg = add(add(add(s7, s9), add(s11, s13)), add(s15, s17));
+    rho = add(add(f[0], sax), sdg);
+    j[0] = add(sub(f[1], f[2]), add(add(d7, d9), add(d11, d13)));
+    j[1] = add(sub(f[3], f[4]), add(sub(d7, d9), add(d15, d17)));
+    j[2] = add(sub(f[5], f[6]), add(sub(d11, d13), sub(d15, d17)));
 }
 
-// Where collide_core reads a node's inputs: f(q) is population q = 19 l + i
-// of the node, psa(i) / psb(i) the densities rho_A / rho_B of neighbour
-// x + c_i in the padded psi field.
+// The float `bytes` beyond a base that is the same for the whole grid: a
+// 32-bit offset per thread, so that the address needs no 64-bit arithmetic
+// (which shares the pipe of the generator's products). A population has
+// fewer than 2^32 / 38 nodes and a padded field fewer than 2^30.
+__device__ __forceinline__ const float* at(const float* base, uint32_t bytes)
+{
+    return reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + bytes);
+}
+__device__ __forceinline__ float* at(float* base, uint32_t bytes)
+{
+    return reinterpret_cast<float*>(reinterpret_cast<char*>(base) + bytes);
+}
+
+// Where collide_core reads a node's inputs: f(i) is population i of both
+// components, psi(i) the densities of neighbour x + c_i in the padded psi
+// field with the components exchanged (x: rho_B, y: rho_A), as the Shan-Chen
+// force of each component takes the other's.
 struct GlobalInputs {
-    const float* __restrict__ fin;  // current populations; (l, i) of node m at m + P.dirN[19 l + i]
-    const float* __restrict__ pA;   // psi_A at the node (padded field); psi_B at pA + padn
-    uint32_t n;
-    long long padn;
-    int sy, sz;                      // padded row and plane strides
+    const float* __restrict__ fin;   // current populations; (l, i) of node m at m + P.dirN[19 l + i]
+    const float* __restrict__ psiA;  // padded fields of rho_A and rho_B
+    const float* __restrict__ psiB;
+    uint32_t n, p;                   // byte offsets of the node in a population and in a padded field
+    uint32_t sy, sz;                 // padded row and plane strides in bytes
     __device__ __forceinline__ GlobalInputs(const float* f, const float* psi, int x, int y, int z, uint32_t node,
                                             const KParams& P)
-        : fin(f), pA(psi + pad_index(x, y, z, P)), n(node), padn(P.padn), sy(P.px), sz(P.px * P.py)
+        : fin(f), psiA(psi), psiB(psi + P.padn), n(4u * node),
+          p(4u * ((uint32_t)(x + 1) + (uint32_t)P.px * ((uint32_t)(y + 1) + (uint32_t)P.py * (uint32_t)(z + 1)))),
+          sy(4u * (uint32_t)P.px), sz(4u * (uint32_t)P.px * (uint32_t)P.py)
     {
     }
-    __device__ __forceinline__ float f(int q, const KParams& P) const { return __ldg(fin + (n + P.dirN[q])); }
-    __device__ __forceinline__ int off(int i) const { return cxv(i) + sy * cyv(i) + sz * czv(i); }
-    __device__ __forceinline__ float psa(int i) const { return __ldg(pA + off(i)); }
-    __device__ __forceinline__ float psb(int i) const { return __ldg(pA + padn + off(i)); }
+    __device__ __forceinline__ Pair f(int i, const KParams& P) const
+    {
+        return Pair{__ldg(at(fin + P.dirN[i], n)), __ldg(at(fin + P.dirN[19 + i], n))};
+    }
+    __device__ __forceinline__ Pair psi(int i) const
+    {
+        const uint32_t o = p + 4u * (uint32_t)cxv(i) + sy * (uint32_t)cyv(i) + sz * (uint32_t)czv(i);
+        return Pair{__ldg(at(psiB, o)), __ldg(at(psiA, o))};
+    }
 };
 
 // Push targets of the populations of node n = (x, y, z). Population (l, i)
@@ -164,6 +218,25 @@ struct PushFrame {
         const uint32_t push_idx = n + (uint32_t)off + P.dirN[19 * l + i];
         return wall ? back_idx : push_idx;
     }
+    // The same target as a byte offset from the first slot of the pair of
+    // opposite directions i belongs to (directions 2 k - 1 and 2 k; the rest
+    // direction alone), the same for both components.
+    __host__ __device__ __forceinline__ uint32_t target_bytes(uint32_t n, int i, const KParams& P, bool& wall) const
+    {
+        const int cx = cxv(i), cy = cyv(i), cz = czv(i);
+        const uint32_t need_p = (cx > 0 ? 1u : 0u) | (cy > 0 ? 2u : 0u) | (cz > 0 ? 4u : 0u);
+        const uint32_t need_m = (cx < 0 ? 1u : 0u) | (cy < 0 ? 2u : 0u) | (cz < 0 ? 4u : 0u);
+        wall = ((wallp & need_p) | (wallm & need_m)) != 0u;
+        const uint32_t N = P.dirN[1];
+        int off = 0;
+        if (cx) off += cx > 0 ? offp[0] : offm[0];
+        if (cy) off += cy > 0 ? offp[1] : offm[1];
+        if (cz) off += cz > 0 ? offp[2] : offm[2];
+        const bool second = i != 0 && i % 2 == 0;
+        const uint32_t push = n + (uint32_t)off + (second ? N : 0u);
+        const uint32_t back = n + (i != 0 && !second ? N : 0u);
+        return 4u * (wall ? back : push);
+    }
 };
 
 // Receiver of the pushed populations for callers that also want the next
@@ -176,39 +249,239 @@ struct NoSink {
     __device__ __forceinline__ void put(int, int, float, bool) {}
 };
 
-// Collision and push-streaming of one fluid node (Eq. (lbe)). With PARTICLE,
-// solid_nb marks the directions whose neighbour is a particle node; their
-// links take the moving rule and feed acc = (F[3], T[3], ledger[2]). TAU1:
-// every relaxation time is 1, so the post-collision modes depend on the
-// input only through rho_l and j_l, and the ghost modes carry noise only.
-// The inputs come from `in` (global memory or a shared-memory tile); the
-// outputs are pushed to fout, population (l, i) of node m at m + P.dirN[19 l + i].
+// sqrt(1 / b_k): the noise amplitude of normalised mode k >= 4 per
+// sqrt(3 kT rho_l) when its relaxation time is 1.
+__device__ constexpr float noise_unit(int k)
+{
+    return k == 4 ? 1.22474487139158905f      // b = 2/3
+           : k == 5 ? 0.866025403784438647f   // 4/3
+           : k == 6 ? 1.5f                    // 4/9
+           : k <= 9 ? 3.0f                    // 1/9
+           : k <= 12 ? 1.22474487139158905f   // 2/3
+           : k <= 15 ? 2.12132034355964257f   // 2/9
+           : k == 16 ? 0.707106781186547524f  // 2
+           : k == 17 ? 0.866025403784438647f  // 4/3
+                     : 1.5f;                  // 4/9
+}
+
+// Adds the thermal noise of a node to its normalised modes n (Eq. (lbe)):
+// per component variance 3 kT rho_l (1 - gamma_k^2) / b_k on mode k >= 4, and
+// an interdiffusion momentum. 33 normals from 9 Philox blocks with counter
+// (step, node, block, 0): A modes 4..18, B modes 4..18, interdiffusion J_x,
+// J_y, J_z. Normals 2p and 2p + 1 come from Box-Muller pair p, pairs 2b and
+// 2b + 1 from block b. B's mode k takes normal k + 11, the second of a pair
+// where A's is the first, so the pairs are formed two at a time, p with
+// p + 8, and B's odd one is kept for the next mode; modes of A and B are then
+// updated together.
+template <bool TAU1>
+__device__ __forceinline__ void add_noise(Pair n[19], Pair rho, float irt, uint32_t node, uint32_t step,
+                                          const KParams& P)
+{
+    const float kt3 = __fmul_rn(3.0f, P.kT);
+    const float rA = fmaxf(rho.x, 0.0f), rB = fmaxf(rho.y, 0.0f);
+    const Pair amp{sqrt_newton(__fmul_rn(kt3, rA)), sqrt_newton(__fmul_rn(kt3, rB))};
+    auto block = [&](int b, uint32_t w[4]) {
+        w[0] = step;
+        w[1] = node;
+        w[2] = (uint32_t)b;
+        w[3] = 0u;
+        philox_rk(w[0], w[1], w[2], w[3], P);
+    };
+    auto mode = [&](int k, float za, float zb) {
+        n[k] = mad(mul(amp, splat(TAU1 ? noise_unit(k) : P.nz_mode[k])), Pair{za, zb}, n[k]);
+    };
+    uint32_t wa[4], wb[4];
+    float z12, z13, z14, left;  // normals 12..14 (A modes 16..18) and 15 (B mode 4)
+    block(3, wa);
+    box_muller2(wa[0], wa[1], wa[2], wa[3], z12, z13, z14, left);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        block(b, wa);
+        block(b + 4, wb);
+#pragma unroll
+        for (int h = 0; h < 4; h += 2) {
+            float a0, a1, b0, b1;
+            box_muller2(wa[h], wa[h + 1], wb[h], wb[h + 1], a0, a1, b0, b1);
+            mode(4 + 4 * b + h, a0, left);
+            mode(5 + 4 * b + h, a1, b0);
+            left = b1;
+        }
+    }
+    float b0, b1, jx, jy, jz, spare;
+    block(7, wa);
+    block(8, wb);
+    box_muller2(wa[0], wa[1], wa[2], wa[3], b0, b1, jx, jy);
+    mode(16, z12, left);
+    mode(17, z13, b0);
+    mode(18, z14, b1);
+    box_muller2(wb[0], wb[1], wb[0], wb[1], jz, spare, jz, spare);
+    const float sJ =
+        __fmul_rn(3.0f * P.nz_j, sqrt_newton(__fmul_rn(__fmul_rn(__fmul_rn(P.kT, rA), rB), fmaxf(irt, 0.0f))));
+    const Pair pm{sJ, -sJ};
+    n[1] = mad(pm, splat(jx), n[1]);
+    n[2] = mad(pm, splat(jy), n[2]);
+    n[3] = mad(pm, splat(jz), n[3]);
+}
+
+// What a node's update takes from its inputs: m the modes of both components
+// (only rho_l and j_l, m[0..3], when every relaxation time is 1), g per axis
+// the Shan-Chen sum 36 sum_i w_i c_i psi(x + c_i) (Eq. (sc-force), omega_i =
+// w_i, psi = rho), the other component's densities for each.
+template <bool TAU1>
+struct NodeState {
+    Pair m[TAU1 ? 4 : 19];
+    Pair g[3];
+};
+
+template <bool TAU1, class In>
+__device__ __forceinline__ void load_modes(const In& in, const KParams& P, NodeState<TAU1>& s)
+{
+    Pair f[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) f[i] = in.f(i, P);
+    if constexpr (TAU1) moments(f, s.m[0], s.m + 1);
+    else to_modes(f, s.m);
+}
+
+// Differences of opposite neighbours first: they are close in value.
+template <bool TAU1, class In>
+__device__ __forceinline__ void load_force(const In& in, NodeState<TAU1>& s)
+{
+    const Pair d1 = sub(in.psi(1), in.psi(2)), d2 = sub(in.psi(3), in.psi(4)), d3 = sub(in.psi(5), in.psi(6));
+    const Pair d7 = sub(in.psi(7), in.psi(8)), d9 = sub(in.psi(9), in.psi(10));
+    const Pair d11 = sub(in.psi(11), in.psi(12)), d13 = sub(in.psi(13), in.psi(14));
+    const Pair d15 = sub(in.psi(15), in.psi(16)), d17 = sub(in.psi(17), in.psi(18));
+    const Pair two = splat(2.0f);
+    s.g[0] = mad(two, d1, add(add(d7, d9), add(d11, d13)));
+    s.g[1] = mad(two, d2, add(sub(d7, d9), add(d15, d17)));
+    s.g[2] = mad(two, d3, add(sub(d11, d13), sub(d15, d17)));
+}
+
+// Collision and push-streaming of one fluid node (Eq. (lbe)) from its loaded
+// state. With PARTICLE, solid_nb marks the directions whose neighbour is a
+// particle node; their links take the moving rule and feed acc = (F[3], T[3],
+// ledger[2]). TAU1: every relaxation time is 1, so the post-collision modes
+// depend on the input only through rho_l and j_l, and the ghost modes carry
+// noise only. The outputs are pushed to fout, population (l, i) of node m at
+// m + P.dirN[19 l + i]. Both components go through packed arithmetic
+// (flbm_pair.h).
 template <bool NOISE, bool PARTICLE, bool TAU1, class In, class Sink = NoSink>
-__device__ __forceinline__ void collide_core(int x, int y, int z, uint32_t n, const In& in,
+__device__ __forceinline__ void collide_push(int x, int y, int z, uint32_t n, const In& in, const NodeState<TAU1>& s,
                                              float* __restrict__ fout, const DevState* __restrict__ st,
                                              const KParams& P, uint32_t solid_nb, double* acc,
                                              Sink* sink = nullptr)
 {
-    float ma[19], mb[19];
-    float rhoA, rhoB;
+    const Pair* m = s.m;
+    const Pair rho = m[0];
+    const float irt = recip_newton(__fadd_rn(rho.x, rho.y));
+
+    // Each component's force from the other's densities, and the external
+    // force density split by rho_l.
+    Pair F[3], hF[3];
     {
-        float fa[19], fb[19];
-#pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            fa[i] = in.f(i, P);
-            fb[i] = in.f(19 + i, P);
-        }
-        if (TAU1) {
-            moments(fa, ma[0], ma + 1);
-            moments(fb, mb[0], mb + 1);
-        } else {
-            to_modes(fa, ma);
-            to_modes(fb, mb);
-        }
-        rhoA = ma[0];
-        rhoB = mb[0];
+        const Pair gr = mul(splat(__fmul_rn(-P.G, 1.0f / 36.0f)), rho);
+        const Pair share = mul(rho, splat(irt));
+        const float ez = P.counterforce ? __fadd_rn(P.ext[2], st->fc_f) : P.ext[2];
+        F[0] = mad(gr, s.g[0], mul(share, splat(P.ext[0])));
+        F[1] = mad(gr, s.g[1], mul(share, splat(P.ext[1])));
+        F[2] = mad(gr, s.g[2], mul(share, splat(ez)));
     }
-    const float rt = rhoA + rhoB;
+    // Hydrodynamical velocity v^(H) = (sum_l j_l + (F_A + F_B)/2) / rho_tot.
+    float u[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        hF[a] = mul(F[a], splat(0.5f));
+        const Pair jh = add(m[1 + a], hF[a]);
+        u[a] = __fmul_rn(__fadd_rn(jh.x, jh.y), irt);
+    }
+
+    // MRT relaxation of both components in moment space. J = rho_l u + F_l / 2
+    // is the relaxed momentum and T_ab = u_a J_b + u_b F_a / 2 the second
+    // moment of equilibrium plus source.
+    Pair fo[19];
+    {
+        Pair J[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) J[a] = mad(rho, splat(u[a]), hF[a]);
+        const Pair mass = add(rho, Pair{st->delta_f[0], st->delta_f[1]});
+        auto T = [&](int a, int b) { return mad(splat(u[a]), J[b], mul(splat(u[b]), hF[a])); };
+        if constexpr (TAU1 && !NOISE) {
+            // No ghost mode: f_i = w_i (base + 3 c_i.J + 9/2 c_i c_i:T), base =
+            // rho_l + delta_l - 3/2 tr T.
+            const Pair d[3] = {T(0, 0), T(1, 1), T(2, 2)};
+            const Pair base = mad(splat(-1.5f), add(add(d[0], d[1]), d[2]), mass);
+            fo[0] = mul(base, splat(1.0f / 3.0f));
+            const Pair b18 = mul(base, splat(1.0f / 18.0f)), b36 = mul(base, splat(1.0f / 36.0f));
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const Pair e = mad(d[a], splat(0.25f), b18);
+                fo[1 + 2 * a] = mad(J[a], splat(1.0f / 6.0f), e);
+                fo[2 + 2 * a] = mad(J[a], splat(-1.0f / 6.0f), e);
+            }
+            // the directions of the plane of axes a < b start at i: ++, --, +-, -+
+            auto plane = [&](int a, int b, int i) {
+                const Pair e = mad(add(d[a], d[b]), splat(0.125f), b36), m = T(a, b);
+                const Pair ep = mad(m, splat(0.25f), e), em = mad(m, splat(-0.25f), e);
+                const Pair op = add(J[a], J[b]), om = sub(J[a], J[b]);
+                fo[i] = mad(op, splat(1.0f / 12.0f), ep);
+                fo[i + 1] = mad(op, splat(-1.0f / 12.0f), ep);
+                fo[i + 2] = mad(om, splat(1.0f / 12.0f), em);
+                fo[i + 3] = mad(om, splat(-1.0f / 12.0f), em);
+            };
+            plane(0, 1, 7);
+            plane(0, 2, 11);
+            plane(1, 2, 15);
+        } else {
+            Pair k[19];  // normalised modes m_k / b_k
+            k[0] = mass;
+            if constexpr (TAU1) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) k[1 + a] = mul(J[a], splat(3.0f));
+                const Pair xx = T(0, 0), yy = T(1, 1), zz = T(2, 2);
+                const Pair yz = add(yy, zz), tr = add(xx, yz);
+                k[4] = mul(tr, splat(1.5f));
+                k[5] = mad(xx, splat(1.5f), mul(yz, splat(-0.75f)));
+                k[6] = mul(sub(yy, zz), splat(2.25f));
+                k[7] = mul(T(0, 1), splat(9.0f));
+                k[8] = mul(T(1, 2), splat(9.0f));
+                k[9] = mul(T(0, 2), splat(9.0f));
+#pragma unroll
+                for (int q = 10; q < 19; ++q) k[q] = splat(0.0f);
+            } else {
+                // equilibrium and source apart: m_eq + gamma (m - m_eq), and
+                // the source by its (1 + gamma_s) / 2
+                const Pair gs = splat(P.gs), gd = splat(P.gd), gg = splat(P.gg);
+                const Pair h = splat(__fmul_rn(0.5f, __fadd_rn(1.0f, P.gs)));
+                Pair ru[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    ru[a] = mul(rho, splat(u[a]));
+                    const Pair dev = sub(add(m[1 + a], hF[a]), ru[a]);
+                    k[1 + a] = mul(mad(gd, dev, J[a]), splat(3.0f));
+                }
+                Pair eq[6], S[6];
+                auto eqab = [&](int a, int b) { return mul(ru[a], splat(u[b])); };
+                auto sab = [&](int a, int b) { return mad(splat(u[a]), F[b], mul(splat(u[b]), F[a])); };
+                const Pair exx = eqab(0, 0), eyy = eqab(1, 1), ezz = eqab(2, 2);
+                const Pair sxx = sab(0, 0), syy = sab(1, 1), szz = sab(2, 2);
+                const Pair eyz = add(eyy, ezz), syz = add(syy, szz);
+                const Pair two = splat(2.0f);
+                eq[0] = add(exx, eyz); S[0] = add(sxx, syz);
+                eq[1] = sub(mul(two, exx), eyz); S[1] = sub(mul(two, sxx), syz);
+                eq[2] = sub(eyy, ezz); S[2] = sub(syy, szz);
+                eq[3] = eqab(0, 1); S[3] = sab(0, 1);
+                eq[4] = eqab(1, 2); S[4] = sab(1, 2);
+                eq[5] = eqab(0, 2); S[5] = sab(0, 2);
+#pragma unroll
+                for (int q = 0; q < 6; ++q)
+                    k[4 + q] = mul(mad(h, S[q], mad(gs, sub(m[4 + q], eq[q]), eq[q])), splat(1.0f / bnorm(4 + q)));
+#pragma unroll
+                for (int q = 10; q < 19; ++q) k[q] = mul(mul(gg, m[q]), splat(1.0f / bnorm(q)));
+            }
+            if (NOISE) add_noise<TAU1>(k, rho, irt, n, st->step_u32, P);
+            from_modes(k, fo);
+        }
+    }
 
     // Particle links of this node: FP32 sums of force, torque about the node
     // (lever c_i / 2) and mass ledger, moved into the FP64 accumulators once
@@ -224,130 +497,43 @@ __device__ __forceinline__ void collide_core(int x, int y, int z, uint32_t n, co
         for (int a = 0; a < 3; ++a) rnf[a] = (float)rn[a];
     }
 
-    // Shan-Chen force, Eq. (sc-force), omega_i = w_i, psi = rho.
-    float ga[3] = {0.f, 0.f, 0.f}, gb[3] = {0.f, 0.f, 0.f};
-    {
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            const float pa = in.psa(i);
-            const float pb = in.psb(i);
-            const float w = wv(i);
-            if (cxv(i)) { ga[0] += (cxv(i) * w) * pb; gb[0] += (cxv(i) * w) * pa; }
-            if (cyv(i)) { ga[1] += (cyv(i) * w) * pb; gb[1] += (cyv(i) * w) * pa; }
-            if (czv(i)) { ga[2] += (czv(i) * w) * pb; gb[2] += (czv(i) * w) * pa; }
-            if (PARTICLE && (solid_nb >> i & 1u)) {
-                // Reaction on the particle of this pair force (virtual layer).
-                const float mag = P.G * w * (rhoA * pb + rhoB * pa);
-                link_add(lk, mag, cxv(i), cyv(i), czv(i));
-            }
-        }
-    }
-    const float irt = 1.0f / rt;
-    float ext[3] = {P.ext[0], P.ext[1], P.ext[2]};
-    if (P.counterforce) ext[2] += st->fc_f;
-    float FA[3], FB[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        FA[a] = -P.G * rhoA * ga[a] + rhoA * irt * ext[a];
-        FB[a] = -P.G * rhoB * gb[a] + rhoB * irt * ext[a];
-    }
-    // Hydrodynamical velocity v^(H) = (sum_l j_l + (F_A + F_B)/2) / rho_tot.
-    float u[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) u[a] = (ma[1 + a] + mb[1 + a] + 0.5f * (FA[a] + FB[a])) * irt;
-    const float uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-
-    // MRT relaxation of each component in moment space, then n_k = m_k / b_k.
-    auto relax = [&](float* m, float rl, const float* Fl, float delta) {
-        const float uF = u[0] * Fl[0] + u[1] * Fl[1] + u[2] * Fl[2];
-        m[0] = rl + delta;
-        const float meq[6] = {rl * uu, rl * (3.0f * u[0] * u[0] - uu), rl * (u[1] * u[1] - u[2] * u[2]),
-                              rl * u[0] * u[1], rl * u[1] * u[2], rl * u[0] * u[2]};
-        const float S[6] = {2.0f * uF, 2.0f * (3.0f * u[0] * Fl[0] - uF), 2.0f * (u[1] * Fl[1] - u[2] * Fl[2]),
-                            u[0] * Fl[1] + u[1] * Fl[0], u[1] * Fl[2] + u[2] * Fl[1], u[0] * Fl[2] + u[2] * Fl[0]};
-        if (TAU1) {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) m[1 + a] = rl * u[a] + 0.5f * Fl[a];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) m[4 + k] = meq[k] + 0.5f * S[k];
-#pragma unroll
-            for (int k = 10; k < 19; ++k) m[k] = 0.0f;
-        } else {
-            const float h = 0.5f * (1.0f + P.gs);
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                m[1 + a] = rl * u[a] + P.gd * (m[1 + a] + 0.5f * Fl[a] - rl * u[a]) + 0.5f * Fl[a];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) m[4 + k] = meq[k] + P.gs * (m[4 + k] - meq[k]) + h * S[k];
-#pragma unroll
-            for (int k = 10; k < 19; ++k) m[k] *= P.gg;
-        }
-#pragma unroll
-        for (int k = 0; k < 19; ++k) m[k] *= 1.0f / bnorm(k);
-    };
-    relax(ma, rhoA, FA, st->delta_f[0]);
-    relax(mb, rhoB, FB, st->delta_f[1]);
-
-    if (NOISE) {
-        // 33 normals from 9 Philox blocks with counter (step, node, block, 0):
-        // A modes 4..18, B modes 4..18, interdiffusion J_x, J_y, J_z.
-        const float sA = sqrtf(3.0f * P.kT * fmaxf(rhoA, 0.0f));
-        const float sB = sqrtf(3.0f * P.kT * fmaxf(rhoB, 0.0f));
-        const float sJ = 3.0f * P.nz_j * sqrtf(P.kT * fmaxf(rhoA, 0.0f) * fmaxf(rhoB, 0.0f) * fmaxf(irt, 0.0f));
-        const uint32_t stp = st->step_u32;
-#pragma unroll
-        for (int blk = 0; blk < 9; ++blk) {
-            uint32_t r0 = stp, r1 = n, r2 = (uint32_t)blk, r3 = 0u;
-            philox_rk(r0, r1, r2, r3, P);
-            float zn[4];
-            box_muller(r0, r1, zn[0], zn[1]);
-            box_muller(r2, r3, zn[2], zn[3]);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int idx = 4 * blk + q;
-                if (idx < 15) ma[4 + idx] += sA * P.nz_mode[4 + idx] * zn[q];
-                else if (idx < 30) mb[4 + idx - 15] += sB * P.nz_mode[4 + idx - 15] * zn[q];
-                else if (idx < 33) {
-                    ma[1 + idx - 30] += sJ * zn[q];
-                    mb[1 + idx - 30] -= sJ * zn[q];
-                }
-            }
-        }
-    }
-
-    // Per-node offsets and wall flags of the push targets.
+    // Push both components (Eq. (lbe) streaming; halfway bounce-back at
+    // walls; moving link rule at the particle): the same target in each
+    // component's block of populations.
     const PushFrame frame(x, y, z, P);
-
-    // Back-transform and push each component (Eq. (lbe) streaming; halfway
-    // bounce-back at walls; moving link rule at the particle).
+    float* __restrict__ foutB = fout + P.dirN[19];
 #pragma unroll
-    for (int l = 0; l < 2; ++l) {
-        float fo[19];
-        from_modes(l == 0 ? ma : mb, fo);
-        const float rl = l == 0 ? rhoA : rhoB;
-#pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            const int cx = cxv(i), cy = cyv(i), cz = czv(i);
-            if (PARTICLE && (solid_nb >> i & 1u)) {
-                // f_{-i}(x, t+1) = f*_i(x) - 6 w_i rho_l (u_b . c_i), u_b at the link midpoint.
-                const uint32_t back_idx = n + P.dirN[19 * l + oppv(i)];
-                const float r[3] = {rnf[0] + 0.5f * cx, rnf[1] + 0.5f * cy, rnf[2] + 0.5f * cz};
-                const float* V = st->Vf;
-                const float* Om = st->Omf;
-                const float ubc = (V[0] + Om[1] * r[2] - Om[2] * r[1]) * cx +
-                                  (V[1] + Om[2] * r[0] - Om[0] * r[2]) * cy +
-                                  (V[2] + Om[0] * r[1] - Om[1] * r[0]) * cz;
-                const float corr = 6.0f * wv(i) * rl * ubc;
-                const float back = fo[i] - corr;
-                fout[back_idx] = back;
-                link_add(lk, fo[i] + back, cx, cy, cz);
-                lk.led[l] += corr;
-                continue;
-            }
-            bool wall;
-            const uint32_t idx = frame.target(n, l, i, P, wall);
-            fout[idx] = fo[i];
-            if constexpr (Sink::active) sink->put(l, i, fo[i], wall);
+    for (int i = 0; i < 19; ++i) {
+        const int cx = cxv(i), cy = cyv(i), cz = czv(i);
+        if (PARTICLE && (solid_nb >> i & 1u)) {
+            // f_{-i}(x, t+1) = f*_i(x) - 6 w_i rho_l (u_b . c_i), u_b at the
+            // link midpoint; the particle takes the momentum both exchange
+            // and the reaction to the pair force with its virtual layer.
+            const uint32_t back_idx = n + P.dirN[oppv(i)];
+            const float r[3] = {rnf[0] + 0.5f * cx, rnf[1] + 0.5f * cy, rnf[2] + 0.5f * cz};
+            const float* V = st->Vf;
+            const float* Om = st->Omf;
+            const float ubc = (V[0] + Om[1] * r[2] - Om[2] * r[1]) * cx + (V[1] + Om[2] * r[0] - Om[0] * r[2]) * cy +
+                              (V[2] + Om[0] * r[1] - Om[1] * r[0]) * cz;
+            const Pair corr = mul(rho, splat(6.0f * wv(i) * ubc));
+            const Pair back = sub(fo[i], corr);
+            fout[back_idx] = back.x;
+            foutB[back_idx] = back.y;
+            const Pair pn = in.psi(i);
+            const Pair ex = add(fo[i], back);
+            link_add(lk, (ex.x + ex.y) + P.G * wv(i) * (rho.x * pn.x + rho.y * pn.y), cx, cy, cz);
+            lk.led[0] += corr.x;
+            lk.led[1] += corr.y;
+            continue;
+        }
+        bool wall;
+        const uint32_t to = frame.target_bytes(n, i, P, wall);
+        const int pair = i == 0 ? 0 : (i & 1) ? i : i - 1;
+        *at(fout + P.dirN[pair], to) = fo[i].x;
+        *at(fout + P.dirN[19 + pair], to) = fo[i].y;
+        if constexpr (Sink::active) {
+            sink->put(0, i, fo[i].x, wall);
+            sink->put(1, i, fo[i].y, wall);
         }
     }
     if (PARTICLE && solid_nb) {
@@ -359,6 +545,19 @@ __device__ __forceinline__ void collide_core(int x, int y, int z, uint32_t n, co
         acc[6] += lk.led[0];
         acc[7] += lk.led[1];
     }
+}
+
+// The whole update of a node from one set of inputs.
+template <bool NOISE, bool PARTICLE, bool TAU1, class In, class Sink = NoSink>
+__device__ __forceinline__ void collide_core(int x, int y, int z, uint32_t n, const In& in,
+                                             float* __restrict__ fout, const DevState* __restrict__ st,
+                                             const KParams& P, uint32_t solid_nb, double* acc,
+                                             Sink* sink = nullptr)
+{
+    NodeState<TAU1> s;
+    load_modes(in, P, s);
+    load_force(in, s);
+    collide_push<NOISE, PARTICLE, TAU1>(x, y, z, n, in, s, fout, st, P, solid_nb, acc, sink);
 }
 
 // collide_core with its inputs read from global memory.
@@ -393,12 +592,29 @@ __device__ __forceinline__ void bulk_tile(int bx, int by, int bz, int tx, int ty
     collide_node<NOISE, false, TAU1>(x, y, z, n, fin, fout, psi, st, P, 0u, nullptr);
 }
 
+// Blocks of the bulk launches: part (0 .. kBulkParts - 1) of a tile, its rows
+// ty / kBulkParts * part onwards. With noise two blocks of 128 threads share
+// a tile, seven per SM: 72 registers hold the update without spills (a
+// spilled register's store goes through to L2), and a half block's slot is
+// refilled sooner. Collide of 128x128x512: 459 us, against 478 us for whole
+// tiles at four blocks of 64 registers and 530 us at three of 80. Without
+// noise 64 registers suffice and the four whole tiles are best: 432 us
+// against 447 us.
+template <bool NOISE>
+constexpr int kBulkParts = NOISE ? 2 : 1;
+template <bool NOISE>
+constexpr int kBulkThreads = kThreadsStep / kBulkParts<NOISE>;
+template <bool NOISE>
+constexpr int kBulkBlocks = NOISE ? 7 : 4;  // resident per SM
+
 template <bool NOISE, bool TAU1>
-static __global__ void __launch_bounds__(kThreadsStep, FLBM_BULK_MINBLOCKS)
+static __global__ void __launch_bounds__(kBulkThreads<NOISE>, kBulkBlocks<NOISE>)
     k_collide_bulk(const float* __restrict__ fin, float* __restrict__ fout, const float* __restrict__ psi,
                    const DevState* __restrict__ st, KParams P)
 {
-    bulk_tile<NOISE, TAU1>(blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, threadIdx.y, fin, fout, psi, st, P);
+    constexpr unsigned parts = kBulkParts<NOISE>;
+    bulk_tile<NOISE, TAU1>(blockIdx.x / parts, blockIdx.y, blockIdx.z, threadIdx.x,
+                           threadIdx.y + blockDim.y * (blockIdx.x % parts), fin, fout, psi, st, P);
 }
 
 // Candidate c on one axis -> tile index, or -1. e0 = first coordinate of the
@@ -484,8 +700,10 @@ __device__ __forceinline__ void near_tile(int cx, int cy, int cz, int tx, int ty
     __syncthreads();
 }
 
+// Two blocks per SM (128 registers): the links' code beside the bulk update
+// spills at three (collide class of 64x64x128: 37.5 us against 51.5 us).
 template <bool NOISE, bool TAU1>
-static __global__ void __launch_bounds__(kThreadsStep, TAU1 ? 3 : 2)
+static __global__ void __launch_bounds__(kThreadsStep, 2)
     k_collide_near(const float* __restrict__ fin, float* __restrict__ fout, const float* __restrict__ psi,
                    DevState* __restrict__ st, const uint8_t* __restrict__ masks,
                    double* __restrict__ partials, KParams P)

@@ -110,10 +110,12 @@ struct StagedInputs {
           p_(stage + kTmaFBytes / 4 + (kTmaPY + ty + 1) * kTmaPX + tx + 1)
     {
     }
-    __device__ __forceinline__ float f(int q, const KParams&) const { return f_[q * kTmaTX * kTmaTY]; }
+    __device__ __forceinline__ Pair f(int i, const KParams&) const
+    {
+        return Pair{f_[i * kTmaTX * kTmaTY], f_[(19 + i) * kTmaTX * kTmaTY]};
+    }
     static __device__ __forceinline__ int off(int i) { return cxv(i) + kTmaPX * (cyv(i) + kTmaPY * czv(i)); }
-    __device__ __forceinline__ float psa(int i) const { return p_[off(i)]; }
-    __device__ __forceinline__ float psb(int i) const { return p_[3 * kTmaPY * kTmaPX + off(i)]; }
+    __device__ __forceinline__ Pair psi(int i) const { return Pair{p_[3 * kTmaPY * kTmaPX + off(i)], p_[off(i)]}; }
 };
 
 // Tile t of the plane-tile grid (x fastest, as the grid of k_collide_bulk).
