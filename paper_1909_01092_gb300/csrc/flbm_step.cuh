@@ -405,82 +405,54 @@ __device__ __forceinline__ void collide_push(int x, int y, int z, uint32_t n, co
         for (int a = 0; a < 3; ++a) J[a] = mad(rho, splat(u[a]), hF[a]);
         const Pair mass = add(rho, Pair{st->delta_f[0], st->delta_f[1]});
         auto T = [&](int a, int b) { return mad(splat(u[a]), J[b], mul(splat(u[b]), hF[a])); };
-        if constexpr (TAU1 && !NOISE) {
-            // No ghost mode: f_i = w_i (base + 3 c_i.J + 9/2 c_i c_i:T), base =
-            // rho_l + delta_l - 3/2 tr T.
-            const Pair d[3] = {T(0, 0), T(1, 1), T(2, 2)};
-            const Pair base = mad(splat(-1.5f), add(add(d[0], d[1]), d[2]), mass);
-            fo[0] = mul(base, splat(1.0f / 3.0f));
-            const Pair b18 = mul(base, splat(1.0f / 18.0f)), b36 = mul(base, splat(1.0f / 36.0f));
+        Pair k[19];  // normalised modes m_k / b_k
+        k[0] = mass;
+        if constexpr (TAU1) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) k[1 + a] = mul(J[a], splat(3.0f));
+            const Pair xx = T(0, 0), yy = T(1, 1), zz = T(2, 2);
+            const Pair yz = add(yy, zz), tr = add(xx, yz);
+            k[4] = mul(tr, splat(1.5f));
+            k[5] = mad(xx, splat(1.5f), mul(yz, splat(-0.75f)));
+            k[6] = mul(sub(yy, zz), splat(2.25f));
+            k[7] = mul(T(0, 1), splat(9.0f));
+            k[8] = mul(T(1, 2), splat(9.0f));
+            k[9] = mul(T(0, 2), splat(9.0f));
+#pragma unroll
+            for (int q = 10; q < 19; ++q) k[q] = splat(0.0f);
+        } else {
+            // equilibrium and source apart: m_eq + gamma (m - m_eq), and
+            // the source by its (1 + gamma_s) / 2
+            const Pair gs = splat(P.gs), gd = splat(P.gd), gg = splat(P.gg);
+            const Pair h = splat(__fmul_rn(0.5f, __fadd_rn(1.0f, P.gs)));
+            Pair ru[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                const Pair e = mad(d[a], splat(0.25f), b18);
-                fo[1 + 2 * a] = mad(J[a], splat(1.0f / 6.0f), e);
-                fo[2 + 2 * a] = mad(J[a], splat(-1.0f / 6.0f), e);
+                ru[a] = mul(rho, splat(u[a]));
+                const Pair dev = sub(add(m[1 + a], hF[a]), ru[a]);
+                k[1 + a] = mul(mad(gd, dev, J[a]), splat(3.0f));
             }
-            // the directions of the plane of axes a < b start at i: ++, --, +-, -+
-            auto plane = [&](int a, int b, int i) {
-                const Pair e = mad(add(d[a], d[b]), splat(0.125f), b36), m = T(a, b);
-                const Pair ep = mad(m, splat(0.25f), e), em = mad(m, splat(-0.25f), e);
-                const Pair op = add(J[a], J[b]), om = sub(J[a], J[b]);
-                fo[i] = mad(op, splat(1.0f / 12.0f), ep);
-                fo[i + 1] = mad(op, splat(-1.0f / 12.0f), ep);
-                fo[i + 2] = mad(om, splat(1.0f / 12.0f), em);
-                fo[i + 3] = mad(om, splat(-1.0f / 12.0f), em);
-            };
-            plane(0, 1, 7);
-            plane(0, 2, 11);
-            plane(1, 2, 15);
-        } else {
-            Pair k[19];  // normalised modes m_k / b_k
-            k[0] = mass;
-            if constexpr (TAU1) {
+            Pair eq[6], S[6];
+            auto eqab = [&](int a, int b) { return mul(ru[a], splat(u[b])); };
+            auto sab = [&](int a, int b) { return mad(splat(u[a]), F[b], mul(splat(u[b]), F[a])); };
+            const Pair exx = eqab(0, 0), eyy = eqab(1, 1), ezz = eqab(2, 2);
+            const Pair sxx = sab(0, 0), syy = sab(1, 1), szz = sab(2, 2);
+            const Pair eyz = add(eyy, ezz), syz = add(syy, szz);
+            const Pair two = splat(2.0f);
+            eq[0] = add(exx, eyz); S[0] = add(sxx, syz);
+            eq[1] = sub(mul(two, exx), eyz); S[1] = sub(mul(two, sxx), syz);
+            eq[2] = sub(eyy, ezz); S[2] = sub(syy, szz);
+            eq[3] = eqab(0, 1); S[3] = sab(0, 1);
+            eq[4] = eqab(1, 2); S[4] = sab(1, 2);
+            eq[5] = eqab(0, 2); S[5] = sab(0, 2);
 #pragma unroll
-                for (int a = 0; a < 3; ++a) k[1 + a] = mul(J[a], splat(3.0f));
-                const Pair xx = T(0, 0), yy = T(1, 1), zz = T(2, 2);
-                const Pair yz = add(yy, zz), tr = add(xx, yz);
-                k[4] = mul(tr, splat(1.5f));
-                k[5] = mad(xx, splat(1.5f), mul(yz, splat(-0.75f)));
-                k[6] = mul(sub(yy, zz), splat(2.25f));
-                k[7] = mul(T(0, 1), splat(9.0f));
-                k[8] = mul(T(1, 2), splat(9.0f));
-                k[9] = mul(T(0, 2), splat(9.0f));
+            for (int q = 0; q < 6; ++q)
+                k[4 + q] = mul(mad(h, S[q], mad(gs, sub(m[4 + q], eq[q]), eq[q])), splat(1.0f / bnorm(4 + q)));
 #pragma unroll
-                for (int q = 10; q < 19; ++q) k[q] = splat(0.0f);
-            } else {
-                // equilibrium and source apart: m_eq + gamma (m - m_eq), and
-                // the source by its (1 + gamma_s) / 2
-                const Pair gs = splat(P.gs), gd = splat(P.gd), gg = splat(P.gg);
-                const Pair h = splat(__fmul_rn(0.5f, __fadd_rn(1.0f, P.gs)));
-                Pair ru[3];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    ru[a] = mul(rho, splat(u[a]));
-                    const Pair dev = sub(add(m[1 + a], hF[a]), ru[a]);
-                    k[1 + a] = mul(mad(gd, dev, J[a]), splat(3.0f));
-                }
-                Pair eq[6], S[6];
-                auto eqab = [&](int a, int b) { return mul(ru[a], splat(u[b])); };
-                auto sab = [&](int a, int b) { return mad(splat(u[a]), F[b], mul(splat(u[b]), F[a])); };
-                const Pair exx = eqab(0, 0), eyy = eqab(1, 1), ezz = eqab(2, 2);
-                const Pair sxx = sab(0, 0), syy = sab(1, 1), szz = sab(2, 2);
-                const Pair eyz = add(eyy, ezz), syz = add(syy, szz);
-                const Pair two = splat(2.0f);
-                eq[0] = add(exx, eyz); S[0] = add(sxx, syz);
-                eq[1] = sub(mul(two, exx), eyz); S[1] = sub(mul(two, sxx), syz);
-                eq[2] = sub(eyy, ezz); S[2] = sub(syy, szz);
-                eq[3] = eqab(0, 1); S[3] = sab(0, 1);
-                eq[4] = eqab(1, 2); S[4] = sab(1, 2);
-                eq[5] = eqab(0, 2); S[5] = sab(0, 2);
-#pragma unroll
-                for (int q = 0; q < 6; ++q)
-                    k[4 + q] = mul(mad(h, S[q], mad(gs, sub(m[4 + q], eq[q]), eq[q])), splat(1.0f / bnorm(4 + q)));
-#pragma unroll
-                for (int q = 10; q < 19; ++q) k[q] = mul(mul(gg, m[q]), splat(1.0f / bnorm(q)));
-            }
-            if (NOISE) add_noise<TAU1>(k, rho, irt, n, st->step_u32, P);
-            from_modes(k, fo);
+            for (int q = 10; q < 19; ++q) k[q] = mul(mul(gg, m[q]), splat(1.0f / bnorm(q)));
         }
+        if (NOISE) add_noise<TAU1>(k, rho, irt, n, st->step_u32, P);
+        from_modes(k, fo);
     }
 
     // Particle links of this node: FP32 sums of force, torque about the node
