@@ -460,31 +460,43 @@ __host__ __device__ __forceinline__ double rel_axis(double r, double X, int L, i
     return d;
 }
 
-// Block-wide sum of 8 doubles into out[0..7] (thread 0 holds the result in
-// s_out). Fixed reduction tree: deterministic.
+// Block-wide sum of 8 doubles into s_out[0..7]. Fixed reduction tree:
+// deterministic. The warp's part is a transposed butterfly: with each
+// exchange a lane hands over half of the values it holds and keeps the sums
+// of the other half, so a lane adds 4 + 2 + 1 + 1 + 1 times instead of the 40
+// of eight separate butterflies (a warp's FP64 addition takes about 16 clocks
+// of the SM's only FP64 pipe).
 // A thread may pass active = false when all its v are 0: warps with no active
-// thread then skip their shuffles (FP64 arithmetic is a slow pipe).
+// thread then skip their shuffles.
 template <int NT>
-__device__ __forceinline__ void block_sum8(double v[8], double* s_red, double* s_out, bool active = true)
+__device__ __forceinline__ void block_sum8(const double v[8], double* s_red, double* s_out, bool active = true)
 {
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int lane = tid & 31, warp = tid >> 5;
     const int nwarp = (blockDim.x * blockDim.y + 31) >> 5;
     const bool warp_any = __any_sync(0xffffffffu, active);
+    // Value of the lane after the exchanges over lane bits 4, 3 and 2.
+    const int k = (lane >> 4 & 1) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1);
+    double a = 0.0;
+    if (warp_any) {
+        const bool u4 = lane & 16, u3 = lane & 8, u2 = lane & 4;
+        double p[4], q[2];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        double a = v[k];
-        if (warp_any) {
+        for (int i = 0; i < 4; ++i)
+            p[i] = (u4 ? v[4 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, u4 ? v[i] : v[4 + i], 16);
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-        }
-        if (lane == 0) s_red[warp * 8 + k] = a;
+        for (int i = 0; i < 2; ++i)
+            q[i] = (u3 ? p[2 + i] : p[i]) + __shfl_xor_sync(0xffffffffu, u3 ? p[i] : p[2 + i], 8);
+        a = (u2 ? q[1] : q[0]) + __shfl_xor_sync(0xffffffffu, u2 ? q[0] : q[1], 4);
+        a += __shfl_xor_sync(0xffffffffu, a, 2);
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
     }
+    if ((lane & 3) == 0) s_red[warp * 8 + k] = a;
     __syncthreads();
     if (tid < 8) {
-        double a = 0.0;
-        for (int w = 0; w < nwarp; ++w) a += s_red[w * 8 + tid];
-        s_out[tid] = a;
+        double t = 0.0;
+        for (int w = 0; w < nwarp; ++w) t += s_red[w * 8 + tid];
+        s_out[tid] = t;
     }
     __syncthreads();
 }
