@@ -241,11 +241,10 @@ struct flbm_ens {
         int max_blocks = 0;
     };
     std::vector<RepLaunch> rep_launches[4];
-    double* obs_tiles = nullptr;
-    double* obs_out = nullptr;
-    double* obs_mode_tiles = nullptr;
-    double* obs_mode_out = nullptr;
-    long long max_tiles = 0;
+    double* obs_parts = nullptr;   // for the replica with the most blocks of k_obs
+    int* obs_marked = nullptr;
+    ObsOut* obs_out = nullptr;
+    long long obs_blocks = 0;
     int cur = 0;                   // all replicas read f[cur] in the next step
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     int64_t graph_launches[2] = {0, 0};
@@ -421,15 +420,14 @@ int allocate(flbm_ens* e)
         at[r] = off;
         off += 2 * sz[r].f + sz[r].psi + sz[r].masks + sz[r].partials + sz[r].counts + sz[r].parts;
         e->nodes += k0.N;
-        e->max_tiles = std::max({e->max_tiles, tile_count(k0), tile_count(k1)});
+        e->obs_blocks = std::max({e->obs_blocks, obs_geom(k0).blocks, obs_geom(k1).blocks});
     }
     if (cudaMalloc(&e->arena, off) != cudaSuccess) return efail(e, FLBM_E_NOMEM, "ensemble state");
     ECK(e, cudaMemsetAsync(e->arena, 0, off, e->stream));
     if (cudaMalloc(&e->d_reps, sizeof(RepDesc) * e->n) != cudaSuccess ||
-        cudaMalloc(&e->obs_tiles, sizeof(double) * 8 * e->max_tiles) != cudaSuccess ||
-        cudaMalloc(&e->obs_out, sizeof(double) * 8) != cudaSuccess ||
-        cudaMalloc(&e->obs_mode_tiles, sizeof(double) * kObsModes * e->max_tiles) != cudaSuccess ||
-        cudaMalloc(&e->obs_mode_out, sizeof(double) * kObsModes) != cudaSuccess)
+        cudaMalloc(&e->obs_parts, sizeof(double) * kObsValues * e->obs_blocks) != cudaSuccess ||
+        cudaMalloc(&e->obs_marked, sizeof(int) * e->obs_blocks) != cudaSuccess ||
+        cudaMalloc(&e->obs_out, sizeof(ObsOut)) != cudaSuccess)
         return efail(e, FLBM_E_NOMEM, "ensemble descriptors");
     char* base = static_cast<char*>(e->arena);
     e->d_states = reinterpret_cast<DevState*>(base);
@@ -716,24 +714,11 @@ int flbm_ensemble_observables(flbm_ens_t* e, int32_t r, flbm_obs* out)
     if (!e || !out || r < 0 || r >= e->n) return efail(e, FLBM_E_INVAL, "invalid argument");
     const KParams& k = e->kp[r];
     const RepDesc& d = e->rd[r];
-    k_obs_tiles<<<dim3(k.gx, k.gy, k.lz), dim3(k.tx, k.ty, 1), 0, e->stream>>>(d.f[e->cur], d.st, d.masks,
-                                                                               e->obs_tiles, k);
-    if (int rc = elaunch(e, "k_obs_tiles")) return rc;
-    k_obs_final<<<1, 1024, 0, e->stream>>>(e->obs_tiles, tile_count(k), e->obs_out);
-    if (int rc = elaunch(e, "k_obs_final")) return rc;
-    k_obs_modes<<<dim3(k.gx, k.gy, k.lz), dim3(k.tx, k.ty, 1), 0, e->stream>>>(d.f[e->cur], d.st, d.masks,
-                                                                               e->obs_mode_tiles, k);
-    if (int rc = elaunch(e, "k_obs_modes")) return rc;
-    k_obs_final_n<kObsModes><<<1, 1024, 0, e->stream>>>(e->obs_mode_tiles, tile_count(k), e->obs_mode_out);
-    if (int rc = elaunch(e, "k_obs_final_n")) return rc;
-    double v[8], vm[kObsModes];
-    DevState s;
-    ECK(e, cudaMemcpyAsync(v, e->obs_out, sizeof(v), cudaMemcpyDeviceToHost, e->stream));
-    ECK(e, cudaMemcpyAsync(vm, e->obs_mode_out, sizeof(vm), cudaMemcpyDeviceToHost, e->stream));
-    ECK(e, cudaMemcpyAsync(&s, d.st, sizeof(s), cudaMemcpyDeviceToHost, e->stream));
+    ECK(e, launch_observe(d.f[e->cur], d.st, d.masks, e->obs_parts, e->obs_marked, e->obs_out, k, e->stream));
+    ObsOut res;
+    ECK(e, cudaMemcpyAsync(&res, e->obs_out, sizeof(res), cudaMemcpyDeviceToHost, e->stream));
     ECK(e, cudaStreamSynchronize(e->stream));
-    fill_obs(v, s, out);
-    fill_mode_obs(vm, out);
+    fill_obs(res, out);
     return out->nonfinite ? efail(e, FLBM_E_NONFINITE, "non-finite populations") : FLBM_OK;
 }
 
@@ -759,10 +744,9 @@ void flbm_ensemble_destroy(flbm_ens_t* e)
     cudaFree(e->arena);
     cudaFree(e->d_reps);
     cudaFree(e->d_items);
-    cudaFree(e->obs_tiles);
+    cudaFree(e->obs_parts);
+    cudaFree(e->obs_marked);
     cudaFree(e->obs_out);
-    cudaFree(e->obs_mode_tiles);
-    cudaFree(e->obs_mode_out);
     delete e;
 }
 

@@ -10,6 +10,7 @@
 
 #include "flbm.h"
 #include "flbm_kernels.cuh"
+#include "flbm_observe.cuh"
 
 namespace flbm {
 
@@ -167,40 +168,37 @@ inline DevState initial_state(const flbm_params& p, const KParams& k)
     return s;
 }
 
-// Observables record from the reduced sums v (mass A, mass B, momentum,
-// kinetic energy, non-finite count) and the particle record.
-inline void fill_obs(const double v[8], const DevState& s, flbm_obs* out)
+// Observables record from the reduced sums and the particle record; each
+// temperature (definitions at flbm_obs) is a ratio of two sums over the bulk
+// fluid nodes.
+inline void fill_obs(const ObsOut& r, flbm_obs* out)
 {
-    out->mass[0] = v[0];
-    out->mass[1] = v[1];
+    const double* v = r.v;
+    const DevState& s = r.s;
+    out->mass[0] = v[32];
+    out->mass[1] = v[33];
     for (int a = 0; a < 3; ++a) {
-        out->momentum[a] = v[2 + a];
+        out->momentum[a] = v[42 + a];
         out->particle_momentum[a] = s.mp * s.V[a];
     }
-    out->kinetic = v[5];
+    out->kinetic = v[41];
     out->pending_mass[0] = s.delta[0] * (double)s.nfluid;
     out->pending_mass[1] = s.delta[1] * (double)s.nfluid;
     out->nfluid = s.nfluid;
     out->step = s.step;
-    out->nonfinite = (int64_t)v[6];
-}
-
-// Temperatures of the fluctuating modes from the kObsModes sums of
-// k_obs_modes (definitions at flbm_obs): each is a ratio of two sums over the
-// bulk fluid nodes.
-inline void fill_mode_obs(const double vm[kObsModes], flbm_obs* out)
-{
+    out->nonfinite = (int64_t)v[46];
     const double b[19] = {1, 1. / 3, 1. / 3, 1. / 3, 2. / 3, 4. / 3, 4. / 9, 1. / 9, 1. / 9, 1. / 9,
                           2. / 3, 2. / 3, 2. / 3, 2. / 9, 2. / 9, 2. / 9, 2, 4. / 3, 4. / 9};
     for (int l = 0; l < 2; ++l)
         for (int k = 0; k < 19; ++k)
-            out->mode_temp[l][k] = (k >= 4 && vm[30 + l] > 0.0) ? vm[15 * l + k - 4] / (3.0 * b[k] * vm[30 + l]) : 0.0;
-    const double rt = vm[30] + vm[31];
+            out->mode_temp[l][k] =
+                (k >= 4 && v[30 + l] > 0.0) ? v[2 * (k - 4) + l] / (3.0 * b[k] * v[30 + l]) : 0.0;
+    const double rt = v[30] + v[31];
     for (int a = 0; a < 3; ++a) {
-        out->diff_temp[a] = vm[35] > 0.0 ? vm[32 + a] / vm[35] : 0.0;
-        out->mom_temp[a] = rt > 0.0 ? vm[36 + a] / rt : 0.0;
+        out->diff_temp[a] = v[40] > 0.0 ? v[34 + 2 * a] / v[40] : 0.0;
+        out->mom_temp[a] = rt > 0.0 ? v[35 + 2 * a] / rt : 0.0;
     }
-    out->n_bulk = (int64_t)vm[39];
+    out->n_bulk = (int64_t)v[45];
 }
 
 // Checks of a particle record read from a checkpoint file before it goes to

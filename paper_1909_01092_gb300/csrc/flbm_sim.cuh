@@ -43,10 +43,9 @@ struct flbm_sim {
     double* box_parts = nullptr;    // per block of the particle box: cover/uncover sums
     int box_blocks = 0;
     long long ncand = 0;
-    double* obs_tiles = nullptr;
-    double* obs_out = nullptr;
-    double* obs_mode_tiles = nullptr;  // per tile: kObsModes sums of k_obs_modes
-    double* obs_mode_out = nullptr;
+    double* obs_parts = nullptr;   // per block of k_obs: its sums, value by value
+    int* obs_marked = nullptr;     // per block of k_obs: redo in FP64
+    flbm::ObsOut* obs_out = nullptr;
     float* scratch_rho = nullptr;
     DevState* traj_dev = nullptr;  // per-step particle records of flbm_run_host
     size_t traj_cap = 0;
