@@ -132,10 +132,12 @@ void setup_tma(flbm_sim* h)
     h->tma_ok = true;  // available; flbm_use_tma switches it on
 }
 
-// Densities, then the psi shell and the virtual layer (one launch), of the
-// current state into psibuf[cur]. With ev, events ev[0..2] bracket the two
-// kernels.
-int launch_psi(flbm_sim* h, cudaEvent_t* ev = nullptr)
+// Densities, then the psi shell and the virtual layer, of the current state
+// into psibuf[cur]. With ev, events ev[0..2] bracket the densities and the
+// shell. in_step: a collide follows, of which only the near tiles read the
+// virtual layer, so it runs on their stream, beside the shell; otherwise one
+// launch does both.
+int launch_psi(flbm_sim* h, cudaEvent_t* ev = nullptr, bool in_step = false)
 {
     const KParams& k = h->kp;
     float* psi = psi_cur(h);
@@ -150,7 +152,14 @@ int launch_psi(flbm_sim* h, cudaEvent_t* ev = nullptr)
     record(h, ev, 1);
     const int nbs = (int)((shell_count(k) + kThreads - 1) / kThreads);
     const int nbv = virtual_blocks(k);
-    k_shell_virtual<<<nbs + nbv, kThreads, 0, h->stream>>>(psi, h->st, h->masks, k, nbs);
+    const bool beside = in_step && nbv > 0;
+    if (beside) {
+        CK(h, cudaEventRecord(h->psi_ev, h->stream));
+        CK(h, cudaStreamWaitEvent(h->side, h->psi_ev, 0));
+        k_shell_virtual<<<nbv, kThreads, 0, h->side>>>(psi, h->st, h->masks, k, 0);
+        if (int rc = launch_check(h, "k_shell_virtual")) return rc;
+    }
+    k_shell_virtual<<<nbs + (beside ? 0 : nbv), kThreads, 0, h->stream>>>(psi, h->st, h->masks, k, nbs);
     if (int rc = launch_check(h, "k_shell_virtual")) return rc;
     record(h, ev, 2);
     h->psi_valid = true;
@@ -221,15 +230,13 @@ int launch_collide(flbm_sim* h, bool fused)
     return FLBM_OK;
 }
 
-// Particle kernels after the collide (the particle update ran in the near
+// Particle kernel after the collide (the particle update ran in the near
 // kernel's last block): next-position masks, cover/uncover and the step's
 // bookkeeping; without a particle only the bookkeeping.
 int launch_particle(flbm_sim* h)
 {
     const KParams& k = h->kp;
     if (k.has_particle) {
-        k_mark_next<<<h->box_blocks, 256, 0, h->stream>>>(h->st, h->masks, h->box_counts, k);
-        if (int rc = launch_check(h, "k_mark_next")) return rc;
         k_cover<<<h->box_blocks, 256, 0, h->stream>>>(h->fbuf[1 - h->cur], h->st, h->masks, h->box_parts,
                                                        h->box_counts, k);
         if (int rc = launch_check(h, "k_cover")) return rc;
@@ -246,7 +253,7 @@ int launch_step(flbm_sim* h, cudaEvent_t* ev = nullptr)
 {
     const KParams& k = h->kp;
     if (!use_fused(h)) {
-        if (int rc = launch_psi(h, ev)) return rc;
+        if (int rc = launch_psi(h, ev, true)) return rc;
         if (int rc = launch_collide(h, false)) return rc;
         record(h, ev, 3);
         if (int rc = launch_particle(h)) return rc;
@@ -511,6 +518,7 @@ int flbm_create(const flbm_params* p, void* f_dev, size_t f_dev_bytes, void* str
         int lo = 0, hi = 0;
         if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
             cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, hi) != cudaSuccess ||
+            cudaEventCreateWithFlags(&h->psi_ev, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&h->join_ev, cudaEventDisableTiming) != cudaSuccess)
             return bail(FLBM_E_CUDA);
@@ -908,6 +916,7 @@ void flbm_destroy(flbm_t* h)
         cudaStreamSynchronize(h->side);
         cudaStreamDestroy(h->side);
     }
+    if (h->psi_ev) cudaEventDestroy(h->psi_ev);
     if (h->fork_ev) cudaEventDestroy(h->fork_ev);
     if (h->join_ev) cudaEventDestroy(h->join_ev);
     delete[] h->traj_host;

@@ -323,6 +323,8 @@ __host__ __device__ __forceinline__ uint32_t solid_neighbours(int x, int y, int 
         hi[a] = P.wall[a] && c[a] == L[a] - 1;
     }
     const unsigned B = (unsigned)P.B;
+    // Every direction's mask byte is loaded (entry 0 where there is none), so
+    // that the 18 loads are in flight together: the node waits for one.
     uint32_t bits = 0u;
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
@@ -336,7 +338,9 @@ __host__ __device__ __forceinline__ uint32_t solid_neighbours(int x, int y, int 
             if (!P.wall[a]) t = t >= L[a] ? t - L[a] : (t < 0 ? t + L[a] : t);
             e[a] = (unsigned)t;
         }
-        if (ok && e[0] < B && e[1] < B && e[2] < B && mask[e[0] + B * (e[1] + B * e[2])]) bits |= 1u << i;
+        ok = ok && e[0] < B && e[1] < B && e[2] < B;
+        const uint8_t in = mask[ok ? e[0] + B * (e[1] + B * e[2]) : 0u];
+        if (ok && in) bits |= 1u << i;
     }
     return bits;
 }
@@ -460,42 +464,81 @@ __host__ __device__ __forceinline__ double rel_axis(double r, double X, int L, i
     return d;
 }
 
+// Sums over the warp of eight doubles a lane, by a transposed butterfly: with
+// each exchange a lane hands over half of the values it holds and keeps the
+// sums of the other half, so a lane adds 4 + 2 + 1 + 1 + 1 times instead of
+// the 40 of eight separate butterflies (a warp's FP64 addition takes about 16
+// clocks of the SM's only FP64 pipe). Returns the sum of value
+// warp_slot(lane); lane sum_lane(k) holds value k. Fixed order.
+__device__ __forceinline__ int warp_slot(int lane)
+{
+    return (lane >> 4 & 1) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1);
+}
+__device__ __forceinline__ int sum_lane(int k) { return (k >> 2 & 1) * 16 + (k >> 1 & 1) * 8 + (k & 1) * 4; }
+__device__ __forceinline__ double warp_sum8(const double v[8], int lane)
+{
+    const bool u4 = lane & 16, u3 = lane & 8, u2 = lane & 4;
+    double p[4], q[2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        p[i] = (u4 ? v[4 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, u4 ? v[i] : v[4 + i], 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) q[i] = (u3 ? p[2 + i] : p[i]) + __shfl_xor_sync(0xffffffffu, u3 ? p[i] : p[2 + i], 8);
+    double a = (u2 ? q[1] : q[0]) + __shfl_xor_sync(0xffffffffu, u2 ? q[0] : q[1], 4);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    return a;
+}
+
 // Block-wide sum of 8 doubles into s_out[0..7]. Fixed reduction tree:
-// deterministic. The warp's part is a transposed butterfly: with each
-// exchange a lane hands over half of the values it holds and keeps the sums
-// of the other half, so a lane adds 4 + 2 + 1 + 1 + 1 times instead of the 40
-// of eight separate butterflies (a warp's FP64 addition takes about 16 clocks
-// of the SM's only FP64 pipe).
-// A thread may pass active = false when all its v are 0: warps with no active
-// thread then skip their shuffles.
+// deterministic. A thread may pass active = false when all its v are 0: warps
+// with no active thread then skip their shuffles.
 template <int NT>
 __device__ __forceinline__ void block_sum8(const double v[8], double* s_red, double* s_out, bool active = true)
 {
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int lane = tid & 31, warp = tid >> 5;
     const int nwarp = (blockDim.x * blockDim.y + 31) >> 5;
-    const bool warp_any = __any_sync(0xffffffffu, active);
-    // Value of the lane after the exchanges over lane bits 4, 3 and 2.
-    const int k = (lane >> 4 & 1) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1);
     double a = 0.0;
-    if (warp_any) {
-        const bool u4 = lane & 16, u3 = lane & 8, u2 = lane & 4;
-        double p[4], q[2];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            p[i] = (u4 ? v[4 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, u4 ? v[i] : v[4 + i], 16);
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-            q[i] = (u3 ? p[2 + i] : p[i]) + __shfl_xor_sync(0xffffffffu, u3 ? p[i] : p[2 + i], 8);
-        a = (u2 ? q[1] : q[0]) + __shfl_xor_sync(0xffffffffu, u2 ? q[0] : q[1], 4);
-        a += __shfl_xor_sync(0xffffffffu, a, 2);
-        a += __shfl_xor_sync(0xffffffffu, a, 1);
-    }
-    if ((lane & 3) == 0) s_red[warp * 8 + k] = a;
+    if (__any_sync(0xffffffffu, active)) a = warp_sum8(v, lane);
+    if ((lane & 3) == 0) s_red[warp * 8 + warp_slot(lane)] = a;
     __syncthreads();
     if (tid < 8) {
         double t = 0.0;
         for (int w = 0; w < nwarp; ++w) t += s_red[w * 8 + tid];
+        s_out[tid] = t;
+    }
+    __syncthreads();
+}
+
+// Block-wide sum of `rows` rows of 8 doubles (written by other blocks) into
+// s_out[0..7], by 256 threads: thread (row r, value k) = (tid / 8, tid % 8)
+// walks rows r, r + 32, ..., then rows add up in a fixed order. Loads of eight
+// rows are in flight together, and rows of zeros, most of them, cost no
+// addition.
+__device__ __forceinline__ void sum_rows8(const double* __restrict__ v, long long rows, double* s_red, double* s_out)
+{
+    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
+    const int lane = tid & 31, warp = tid >> 5;
+    double a = 0.0;
+    for (long long r0 = tid >> 3; r0 < rows; r0 += 256) {
+        double b[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const long long r = r0 + 32 * q;
+            b[q] = r < rows ? __ldcg(v + r * 8 + (tid & 7)) : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (b[q] != 0.0) a += b[q];
+    }
+    a += __shfl_xor_sync(0xffffffffu, a, 8);
+    a += __shfl_xor_sync(0xffffffffu, a, 16);
+    if (lane < 8) s_red[warp * 8 + lane] = a;
+    __syncthreads();
+    if (tid < 8) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += s_red[w * 8 + tid];
         s_out[tid] = t;
     }
     __syncthreads();

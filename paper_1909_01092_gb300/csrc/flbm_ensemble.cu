@@ -13,9 +13,9 @@
 // instead takes the descriptors of up to kChunkReps replicas as a kernel
 // parameter (kb_bulk_rep). The step sequence (densities; density shell;
 // collide-stream of the bulk tiles; on a side stream meanwhile the virtual
-// layer, the near tiles, whose launch ends with each replica's particle
-// update, and the next-position masks; cover/uncover ending with each
-// replica's bookkeeping) is captured into a CUDA graph of two steps when the
+// layer and the near tiles, whose launch ends with each replica's particle
+// update; next-position masks and cover/uncover ending with each replica's
+// bookkeeping) is captured into a CUDA graph of two steps when the
 // stream allows capture.
 #include <cuda_runtime.h>
 
@@ -167,14 +167,6 @@ static __global__ void __launch_bounds__(256, 2)
     FLBM_END_ITEMS
 }
 
-static __global__ void __launch_bounds__(256) kb_mark_next(const RepDesc* __restrict__ reps,
-                                                           const Item* __restrict__ items, int nitems)
-{
-    FLBM_FOR_ITEMS
-    mark_next_block(it.y, sR.st, sR.masks, sR.box_counts, P);
-    FLBM_END_ITEMS
-}
-
 static __global__ void __launch_bounds__(256) kb_cover(const RepDesc* __restrict__ reps,
                                                        const Item* __restrict__ items, int nitems, int par)
 {
@@ -203,8 +195,7 @@ enum WorkKind {
     W_VIRT,            // virtual layer (blocks of kb_shell after the shell's)
     W_BULK,            // + variant (4 lists)
     W_NEAR = W_BULK + 4,  // + variant (4 lists)
-    W_MARK = W_NEAR + 4,
-    W_COVER,
+    W_COVER = W_NEAR + 4,
     W_FINISH,
     W_COUNT
 };
@@ -220,8 +211,7 @@ struct flbm_ens {
     std::vector<RepDesc> rd;
     flbm_ens_config cfg{0, 4, 0};
     cudaStream_t stream = nullptr;
-    // Virtual layers, near-particle collide and next-position masks on a
-    // higher-priority side stream, concurrent with the shells and the bulk
+    // Virtual layers and near-particle collide on a higher-priority side stream, concurrent with the shells and the bulk
     // collide (disjoint writes), forked (psi_ev, fork_ev) and joined by events.
     cudaStream_t side = nullptr;
     cudaEvent_t psi_ev = nullptr, fork_ev = nullptr, join_ev = nullptr;
@@ -286,7 +276,7 @@ long long blocks_of(const KParams& k, int w)
     if (w == W_VIRT) return part ? box_block_count(k) : 0;
     if (w >= W_BULK && w < W_BULK + 4) return variant(k) == w - W_BULK ? tile_count(k) : 0;
     if (w >= W_NEAR && w < W_NEAR + 4) return (part && variant(k) == w - W_NEAR) ? cand_count(k) : 0;
-    if (w == W_MARK || w == W_COVER) return part ? box_block_count(k) : 0;
+    if (w == W_COVER) return part ? box_block_count(k) : 0;
     return part ? 0 : 1;  // W_FINISH: with a particle the cover launch finishes the step
 }
 
@@ -494,8 +484,8 @@ int ens_step(flbm_ens* e)
     if (int rc = launch_list(e, W_DENSITY, kb_density, "kb_density", par)) return rc;
     // The particles' share of the step runs on the side stream: the virtual
     // layers once the densities are in, the near tiles once the shells are
-    // in too, then the next-position masks. The shells and the bulk tiles,
-    // which read neither, run on the main stream meanwhile.
+    // in too. The shells and the bulk tiles, which read neither, run on the
+    // main stream meanwhile.
     const bool near = e->off[W_NEAR + 4] > e->off[W_NEAR];
     if (near) {
         ECK(e, cudaEventRecord(e->psi_ev, e->stream));
@@ -512,7 +502,6 @@ int ens_step(flbm_ens* e)
         if (int rc = launch_on(e, e->side, W_NEAR + 1, kb_near<false, true>, "kb_near", par)) return rc;
         if (int rc = launch_on(e, e->side, W_NEAR + 2, kb_near<true, false>, "kb_near", par)) return rc;
         if (int rc = launch_on(e, e->side, W_NEAR + 3, kb_near<true, true>, "kb_near", par)) return rc;
-        if (int rc = launch_on(e, e->side, W_MARK, kb_mark_next, "kb_mark_next")) return rc;
         ECK(e, cudaEventRecord(e->join_ev, e->side));
     }
     if (e->cfg.ctas_per_sm == 0) {
@@ -524,7 +513,6 @@ int ens_step(flbm_ens* e)
         if (int rc = launch_list(e, W_BULK + 3, kb_bulk<true, true>, "kb_bulk", par)) return rc;
     }
     if (near) ECK(e, cudaStreamWaitEvent(e->stream, e->join_ev, 0));
-    else if (int rc = launch_list(e, W_MARK, kb_mark_next, "kb_mark_next")) return rc;
     if (int rc = launch_list(e, W_COVER, kb_cover, "kb_cover", par)) return rc;
     if (int rc = launch_list(e, W_FINISH, kb_finish, "kb_finish")) return rc;
     e->cur = 1 - e->cur;

@@ -10,7 +10,7 @@
 //                     the particle, momentum exchange and Shan-Chen reaction
 //                     reduced per tile (Eq. (lbe)); the near launch's last block
 //                     advances the particle (leap-frog)
-//   k_mark_next, k_cover : particle nodes at the new position, cover/uncover,
+//   k_cover         : particle nodes at the new position, cover/uncover,
 //                     mass-correction ledger; the cover launch's last block
 //                     finishes the step (k_finish without a particle)
 #pragma once

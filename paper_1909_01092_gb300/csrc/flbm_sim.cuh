@@ -71,10 +71,10 @@ struct flbm_sim {
     int tma_grid = 0;
     long long tma_wait = 0;  // limit of its waits for a tile's inputs, SM cycles (set at creation)
     // The near-particle collide runs on a second, higher-priority stream,
-    // concurrently with the bulk collide (they write disjoint populations);
-    // fork and join by events.
+    // concurrently with the bulk collide (they write disjoint populations),
+    // after the virtual layer, which only it reads; fork and join by events.
     cudaStream_t side = nullptr;
-    cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+    cudaEvent_t psi_ev = nullptr, fork_ev = nullptr, join_ev = nullptr;
     long long ntiles = 0;
     int64_t launches = 0;
     int64_t adj_tape_limit = -1;  // flbm_adjoint_tape_limit: < 0 automatic, 0 never, > 0 bytes

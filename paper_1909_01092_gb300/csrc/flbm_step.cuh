@@ -11,12 +11,13 @@
 // Both kernels apply the same tile_near() test, so every tile runs exactly once.
 // The particle update runs in the last block of the near launch (after every
 // candidate's partials are written); the next-position masks and the
-// cover/uncover pass run over the particle box, and the last block of the
-// cover launch does the step's bookkeeping. "Last block" is an atomic ticket
+// cover/uncover pass run over the particle box in one launch, whose last
+// block does the step's bookkeeping. "Last block" is an atomic ticket
 // per launch: no block waits for another.
 #pragma once
 
 #include "flbm_device.cuh"
+#include "flbm_df.h"
 
 namespace flbm {
 
@@ -698,25 +699,36 @@ __host__ __device__ __forceinline__ void box_origin(const double X[3], const KPa
     }
 }
 
+// Is lattice node c strictly inside the sphere around X (FP64)?
+__host__ __device__ __forceinline__ bool node_inside(const int c[3], const double X[3], const KParams& P)
+{
+    const int L[3] = {P.lx, P.ly, P.lz};
+    double s = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double r = rel_axis((double)c[a], X[a], L[a], P.wall[a]);
+        s += r * r;
+    }
+    return s < P.R * P.R;
+}
+
 // Particle node test for box entry t of a box at origin o around centre X (FP64).
 __host__ __device__ __forceinline__ bool box_node_inside(int t, const int o[3], const double X[3], const KParams& P)
 {
     const int B = P.B;
     const int d[3] = {t % B, (t / B) % B, t / (B * B)};
     const int L[3] = {P.lx, P.ly, P.lz};
-    double s = 0.0;
+    int c[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        int c = o[a] + d[a];
+        c[a] = o[a] + d[a];
         if (P.wall[a]) {
-            if (c < 0 || c >= L[a]) return false;
-        } else if (c >= L[a]) {
-            c -= L[a];
+            if (c[a] < 0 || c[a] >= L[a]) return false;
+        } else if (c[a] >= L[a]) {
+            c[a] -= L[a];
         }
-        const double r = rel_axis((double)c, X[a], L[a], P.wall[a]);
-        s += r * r;
     }
-    return s < P.R * P.R;
+    return node_inside(c, X, P);
 }
 
 // ---------------------------------------------------------------------------
@@ -728,34 +740,37 @@ __device__ __forceinline__ void update_particle(DevState* __restrict__ st, const
 {
     __shared__ double s_red[(256 / 32) * 8];
     __shared__ double s_out[8];
-    const long long ncand = (long long)P.ncx * P.ncy * P.ncz;
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    const int nthr = blockDim.x * blockDim.y;
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long c = tid; c < ncand; c += nthr)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += __ldcg(partials + c * 8 + k);
-    block_sum8<256>(acc, s_red, s_out);
+    // The record's values are loaded before the sum, which their latency then
+    // overlaps.
+    const int a = tid;
+    double Pp = 0.0, Lp = 0.0, v0 = 0.0, om0 = 0.0, x0 = 0.0, ext = 0.0;
+    if (a < 3) {
+        Pp = st->Ppend[a];
+        Lp = st->Lpend[a];
+        v0 = st->V[a];
+        om0 = st->Om[a];
+        x0 = st->X[a];
+        ext = (a == 2) ? st->Fp : 0.0;
+    }
+    sum_rows8(partials, (long long)P.ncx * P.ncy * P.ncz, s_red, s_out);
     // One thread per axis: the three components are independent. FP64 on a
     // part whose FP64 is slow, so products with 1 / m_p and 1 / I_p, and the
     // periodic wrap as a conditional shift (floor only for a longer step).
-    const int a = tid;
     if (a >= 3) return;
     const int L = a == 0 ? P.lx : (a == 1 ? P.ly : P.lz);
-    const double F = s_out[a] + st->Ppend[a];
-    const double T = s_out[3 + a] + st->Lpend[a];
+    const double F = s_out[a] + Pp;
+    const double T = s_out[3 + a] + Lp;
     st->F[a] = F;
     st->T[a] = T;
-    const double ext = (a == 2) ? st->Fp : 0.0;
-    const double v0 = st->V[a];
     const double vn = v0 + (F + ext) * P.inv_mp;
     st->Vavg[a] = 0.5 * (v0 + vn);
     st->V[a] = vn;
-    const double om = st->Om[a] + T * P.inv_Ip;
+    const double om = om0 + T * P.inv_Ip;
     st->Om[a] = om;
     st->Vf[a] = (float)vn;
     st->Omf[a] = (float)om;
-    double xn = st->X[a] + vn;
+    double xn = x0 + vn;
     if (!P.wall[a]) {
         if (xn >= L) xn -= L;
         else if (xn < 0.0) xn += L;
@@ -775,58 +790,62 @@ __device__ __forceinline__ void update_particle(DevState* __restrict__ st, const
     st->box_next[a] = o;
 }
 
-// (2) Particle nodes at the new position -> mask[1 - cur]; per-block counts.
-// Block blk of 256 box entries.
-__device__ __forceinline__ void mark_next_block(int blk, const DevState* __restrict__ st, uint8_t* __restrict__ masks,
-                                                int* __restrict__ counts, const KParams& P)
-{
-    __shared__ int s_cnt[256 / 32];
-    const int B3 = P.B * P.B * P.B;
-    const int t = blk * 256 + threadIdx.x;
-    const int o[3] = {st->box_next[0], st->box_next[1], st->box_next[2]};
-    const double X[3] = {st->X[0], st->X[1], st->X[2]};
-    int in = 0;
-    if (t < B3) {
-        in = box_node_inside(t, o, X, P) ? 1 : 0;
-        masks[(size_t)(1 - st->cur) * B3 + t] = (uint8_t)in;
-    }
-    int c = __reduce_add_sync(0xffffffffu, in);
-    if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int a = 0;
-        for (int w = 0; w < 256 / 32; ++w) a += s_cnt[w];
-        counts[blk] = a;
-    }
-    __syncthreads();
-}
-
-static __global__ void __launch_bounds__(256) k_mark_next(const DevState* __restrict__ st, uint8_t* __restrict__ masks,
-                                                          int* __restrict__ counts, KParams P)
-{
-    mark_next_block(blockIdx.x, st, masks, counts, P);
-}
-
-// (3) Cover (new box) and uncover (old box) on the post-stream populations f;
-// per-block FP64 partials of impulse, angular impulse and mass ledger.
-// Exact FP64 sum of the 19 float populations of component l at node m
-// (exact: populations are floats of similar magnitude, so every partial sum
-// fits in a double and the order does not matter); four chains to shorten
-// the dependent FP64 additions, which are slow on this part.
+// Exact sum of the 19 float populations of component l at node m: floats of
+// similar magnitude, whose sums fit the 48 bits of a double-float (and do so
+// in any order), so the slow FP64 pipe only sees the result.
 __device__ __forceinline__ double pop_sum(const float* __restrict__ f, int l, long long m, long long N)
 {
-    double s4[4] = {0.0, 0.0, 0.0, 0.0};
+    float v[19];
 #pragma unroll
-    for (int i = 0; i < 19; ++i) s4[i & 3] += (double)f[(long long)(19 * l + i) * N + m];
-    return (s4[0] + s4[1]) + (s4[2] + s4[3]);
+    for (int i = 0; i < 19; ++i) v[i] = f[(long long)(19 * l + i) * N + m];
+    df s(v[0]);
+#pragma unroll
+    for (int i = 1; i < 19; ++i) s = s + v[i];
+    return s.value();
 }
 
+// c_i along axis a for a direction known at run time: +1, 0 or -1.
+__device__ __forceinline__ int dir_of(int i, int a)
+{
+    constexpr uint32_t p[3] = {1u << 1 | 1u << 7 | 1u << 9 | 1u << 11 | 1u << 13,
+                               1u << 3 | 1u << 7 | 1u << 10 | 1u << 15 | 1u << 17,
+                               1u << 5 | 1u << 11 | 1u << 14 | 1u << 15 | 1u << 18};
+    constexpr uint32_t m[3] = {1u << 2 | 1u << 8 | 1u << 10 | 1u << 12 | 1u << 14,
+                               1u << 4 | 1u << 8 | 1u << 9 | 1u << 16 | 1u << 18,
+                               1u << 6 | 1u << 12 | 1u << 13 | 1u << 16 | 1u << 17};
+    const uint32_t pa = a == 0 ? p[0] : (a == 1 ? p[1] : p[2]), ma = a == 0 ? m[0] : (a == 1 ? m[1] : m[2]);
+    return (int)(pa >> i & 1u) - (int)(ma >> i & 1u);
+}
+__device__ __forceinline__ double signed_by(int s, double v) { return s == 0 ? 0.0 : (s > 0 ? v : -v); }
+
+// Component k of (p, r x p, mass): lane k's share of what an event at r gives.
+__device__ __forceinline__ double event_value(int k, const double r[3], const double p[3], double mA, double mB)
+{
+    const int a = k >= 3 ? k - 3 : k;
+    const double rb = a == 0 ? r[1] : (a == 1 ? r[2] : r[0]), rc = a == 0 ? r[2] : (a == 1 ? r[0] : r[1]);
+    const double pb = a == 0 ? p[1] : (a == 1 ? p[2] : p[0]), pc = a == 0 ? p[2] : (a == 1 ? p[0] : p[1]);
+    const double cross = rb * pc - rc * pb;
+    const double lin = k == 0 ? p[0] : (k == 1 ? p[1] : p[2]);
+    return k < 3 ? lin : (k < 6 ? cross : (k == 6 ? mA : mB));
+}
+
+// (2) Particle nodes at the new position -> mask[1 - cur] and their count,
+// cover (new box) and uncover (old box) on the post-stream populations f;
+// per-block FP64 partials of impulse, angular impulse and mass ledger. Block
+// blk of 256 box entries. No thread reads what another marks: where a node's
+// new state is asked it is tested again.
+//
+// The events of a warp's entries are taken one after the other by the whole
+// warp: its lanes share the populations, the neighbours and the axes, and lane
+// k keeps the k-th of the eight sums. One thread per event held the step's
+// critical path for 8 to 10 us of chained FP64.
 __device__ __forceinline__ void cover_block(int blk, float* __restrict__ f, const DevState* __restrict__ st,
-                                            const uint8_t* __restrict__ masks, double* __restrict__ parts,
-                                            const KParams& P)
+                                            uint8_t* __restrict__ masks, int* __restrict__ counts,
+                                            double* __restrict__ parts, const KParams& P)
 {
     __shared__ double s_red[(256 / 32) * 8];
-    __shared__ double s_out[8];
+    __shared__ int s_cnt[256 / 32];
+    __shared__ int s_any;
     const int B = P.B;
     const int B3 = B * B * B;
     const int t = blk * 256 + threadIdx.x;
@@ -834,68 +853,83 @@ __device__ __forceinline__ void cover_block(int blk, float* __restrict__ f, cons
     const int cur = st->cur;
     const int o_old[3] = {st->box0[0], st->box0[1], st->box0[2]};
     const int o_new[3] = {st->box_next[0], st->box_next[1], st->box_next[2]};
+    const double X[3] = {st->X[0], st->X[1], st->X[2]};
     const uint8_t* m_old = masks + (size_t)cur * B3;
-    const uint8_t* m_new = masks + (size_t)(1 - cur) * B3;
     const int L[3] = {P.lx, P.ly, P.lz};
     const long long N = P.N;
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    bool uncovered = false;
-    int cu_[3] = {0, 0, 0};  // an uncovered node of this thread
+    if (threadIdx.x == 0) s_any = 0;
+    bool now = false, covered = false, uncovered = false;
+    int cc[3] = {0, 0, 0}, cu_[3] = {0, 0, 0};  // the covered / uncovered node of this thread
     if (t < B3) {
         const int d[3] = {t % B, (t / B) % B, t / (B * B)};
-        if (m_new[t]) {  // covered: particle node now, fluid before
-            int c[3];
+        const bool was = m_old[t] != 0;
+        now = box_node_inside(t, o_new, X, P);
+        masks[(size_t)(1 - cur) * B3 + t] = (uint8_t)now;
+        if (now) {
             for (int a = 0; a < 3; ++a) {
-                c[a] = o_new[a] + d[a];
-                if (!P.wall[a] && c[a] >= L[a]) c[a] -= L[a];
+                cc[a] = o_new[a] + d[a];
+                if (!P.wall[a] && cc[a] >= L[a]) cc[a] -= L[a];
             }
-            if (!is_solid(c[0], c[1], c[2], o_old, m_old, P)) {
-                const long long n = c[0] + (long long)P.lx * (c[1] + (long long)P.ly * c[2]);
-                double j4[3][4] = {}, r4[2][4] = {};  // exact sums in four chains
-                for (int l = 0; l < 2; ++l)
-#pragma unroll
-                    for (int i = 0; i < 19; ++i) {
-                        const double fv = f[(long long)(19 * l + i) * N + n];
-                        r4[l][i & 3] += fv;
-                        if (cxv(i)) j4[0][i & 3] += cxv(i) > 0 ? fv : -fv;
-                        if (cyv(i)) j4[1][i & 3] += cyv(i) > 0 ? fv : -fv;
-                        if (czv(i)) j4[2][i & 3] += czv(i) > 0 ? fv : -fv;
-                    }
-                double j[3], rl[2];
-                for (int a = 0; a < 3; ++a) j[a] = (j4[a][0] + j4[a][1]) + (j4[a][2] + j4[a][3]);
-                for (int l = 0; l < 2; ++l) rl[l] = (r4[l][0] + r4[l][1]) + (r4[l][2] + r4[l][3]);
-                double r[3];
-                for (int a = 0; a < 3; ++a) r[a] = rel_axis((double)c[a], st->X[a], L[a], P.wall[a]);
-                acc[0] += j[0]; acc[1] += j[1]; acc[2] += j[2];
-                acc[3] += r[1] * j[2] - r[2] * j[1];
-                acc[4] += r[2] * j[0] - r[0] * j[2];
-                acc[5] += r[0] * j[1] - r[1] * j[0];
-                acc[6] += rl[0];
-                acc[7] += rl[1];
-            }
+            covered = !is_solid(cc[0], cc[1], cc[2], o_old, m_old, P);
         }
-        if (m_old[t]) {  // uncovered: particle node before, fluid now
+        if (was) {
             for (int a = 0; a < 3; ++a) {
                 cu_[a] = o_old[a] + d[a];
                 if (!P.wall[a] && cu_[a] >= L[a]) cu_[a] -= L[a];
             }
-            uncovered = !is_solid(cu_[0], cu_[1], cu_[2], o_new, m_new, P);
+            uncovered = !node_inside(cu_, X, P);
         }
     }
-    // Each uncovered node of the warp in turn, by the whole warp: lane j
-    // (1..18) sums the populations of neighbour j, the warp adds them up
-    // (exact sums), and the lanes write the refilled populations.
-    unsigned um = __ballot_sync(0xffffffffu, uncovered);
+    const unsigned marked = __ballot_sync(0xffffffffu, now);
+    unsigned cm = __ballot_sync(0xffffffffu, covered), um = __ballot_sync(0xffffffffu, uncovered);
+    double acc = 0.0;  // lanes 0..7: the warp's sum of that component
+    const bool events = (cm | um) != 0u;
+    // Covered nodes: lane q holds population q, lanes 0..5 also 32 + q.
+    while (cm) {
+        const int src = __ffs(cm) - 1;
+        cm &= cm - 1;
+        int c[3];
+        for (int a = 0; a < 3; ++a) c[a] = __shfl_sync(0xffffffffu, cc[a], src);
+        const long long n = c[0] + (long long)P.lx * (c[1] + (long long)P.ly * c[2]);
+        const double f0 = f[(long long)lane * N + n];
+        const double f1 = lane < 6 ? (double)f[(long long)(32 + lane) * N + n] : 0.0;
+        const int i0 = lane < 19 ? lane : lane - 19, i1 = 13 + lane;
+        double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            v[a] = signed_by(dir_of(i0, a), f0) + (lane < 6 ? signed_by(dir_of(i1, a), f1) : 0.0);
+        v[3] = lane < 19 ? f0 : 0.0;
+        v[4] = (lane < 19 ? 0.0 : f0) + f1;
+        const double s = warp_sum8(v, lane);
+        double p[3], r[3];
+        double ra = 0.0;
+        if (lane < 3) {
+            const int ca = lane == 0 ? c[0] : (lane == 1 ? c[1] : c[2]);
+            const double Xa = lane == 0 ? X[0] : (lane == 1 ? X[1] : X[2]);
+            const int La = lane == 0 ? L[0] : (lane == 1 ? L[1] : L[2]);
+            ra = rel_axis((double)ca, Xa, La, P.wall[lane]);
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            p[a] = __shfl_sync(0xffffffffu, s, sum_lane(a));
+            r[a] = __shfl_sync(0xffffffffu, ra, a);
+        }
+        const double mA = __shfl_sync(0xffffffffu, s, sum_lane(3)), mB = __shfl_sync(0xffffffffu, s, sum_lane(4));
+        acc += event_value(lane & 7, r, p, mA, mB);
+    }
+    // Uncovered nodes: lane j (1..18) sums the populations of neighbour j,
+    // the warp adds them up (exact sums), and the lanes write the refilled
+    // populations.
     while (um) {
         const int src = __ffs(um) - 1;
         um &= um - 1;
         int c[3];
         for (int a = 0; a < 3; ++a) c[a] = __shfl_sync(0xffffffffu, cu_[a], src);
         double m0 = 0.0, m1 = 0.0;
-        int one = 0;
+        bool ok = false;
         if (lane >= 1 && lane <= 18) {
-            int q[3] = {c[0] + cxv(lane), c[1] + cyv(lane), c[2] + czv(lane)};
-            bool ok = true;
+            int q[3] = {c[0] + dir_of(lane, 0), c[1] + dir_of(lane, 1), c[2] + dir_of(lane, 2)};
+            ok = true;
             for (int a = 0; a < 3; ++a) {
                 if (q[a] < 0 || q[a] >= L[a]) {
                     if (P.wall[a]) ok = false;
@@ -903,49 +937,68 @@ __device__ __forceinline__ void cover_block(int blk, float* __restrict__ f, cons
                 }
             }
             // a fluid neighbour that was fluid before as well
-            if (ok && !is_solid(q[0], q[1], q[2], o_new, m_new, P) && !is_solid(q[0], q[1], q[2], o_old, m_old, P)) {
+            ok = ok && !is_solid(q[0], q[1], q[2], o_old, m_old, P) && !node_inside(q, X, P);
+            if (ok) {
                 const long long m = q[0] + (long long)P.lx * (q[1] + (long long)P.ly * q[2]);
                 m0 = pop_sum(f, 0, m, N);
                 m1 = pop_sum(f, 1, m, N);
-                one = 1;
             }
+        }
+        const int cnt = __popc(__ballot_sync(0xffffffffu, ok));
+        // lanes 0..15 end with component A, lanes 16..31 with B
+        const bool up = lane >= 16;
+        double ms = (up ? m1 : m0) + __shfl_xor_sync(0xffffffffu, up ? m0 : m1, 16);
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) ms += __shfl_xor_sync(0xffffffffu, ms, off);
+        // neighbour-mean densities; the initial densities if no fluid neighbour is left
+        const double rl = cnt ? ms / cnt : (up ? P.rho0[1] : P.rho0[0]);
+        const double rA = __shfl_sync(0xffffffffu, rl, 0), rB = __shfl_sync(0xffffffffu, rl, 16);
+        double r[3], ub[3], ra = 0.0, ua = 0.0;
+        if (lane < 3) {
+            const int ca = lane == 0 ? c[0] : (lane == 1 ? c[1] : c[2]);
+            const double Xa = lane == 0 ? X[0] : (lane == 1 ? X[1] : X[2]);
+            const int La = lane == 0 ? L[0] : (lane == 1 ? L[1] : L[2]);
+            ra = rel_axis((double)ca, Xa, La, P.wall[lane]);
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            m0 += __shfl_xor_sync(0xffffffffu, m0, off);
-            m1 += __shfl_xor_sync(0xffffffffu, m1, off);
-            one += __shfl_xor_sync(0xffffffffu, one, off);
+        for (int a = 0; a < 3; ++a) r[a] = __shfl_sync(0xffffffffu, ra, a);
+        if (lane < 3) {
+            const int b = lane == 2 ? 0 : lane + 1, e = lane == 0 ? 2 : lane - 1;
+            const double rb = b == 0 ? r[0] : (b == 1 ? r[1] : r[2]), re = e == 0 ? r[0] : (e == 1 ? r[1] : r[2]);
+            ua = st->V[lane] + st->Om[b] * re - st->Om[e] * rb;
         }
-        const int cnt = one;
-        // neighbour-mean densities; the initial densities if no fluid neighbour is left
-        const double rls[2] = {cnt ? m0 / cnt : P.rho0[0], cnt ? m1 / cnt : P.rho0[1]};
-        double r[3];
-        for (int a = 0; a < 3; ++a) r[a] = rel_axis((double)c[a], st->X[a], L[a], P.wall[a]);
-        const double ub[3] = {st->V[0] + st->Om[1] * r[2] - st->Om[2] * r[1],
-                              st->V[1] + st->Om[2] * r[0] - st->Om[0] * r[2],
-                              st->V[2] + st->Om[0] * r[1] - st->Om[1] * r[0]};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) ub[a] = __shfl_sync(0xffffffffu, ua, a);
         const long long n = c[0] + (long long)P.lx * (c[1] + (long long)P.ly * c[2]);
-        const double uu = ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2];
+        const double base = 1.0 - 1.5 * (ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]);
         for (int q = lane; q < 38; q += 32) {  // population (l, i) = (q / 19, q % 19)
-            const int l = q / 19, i = q % 19;
-            const double cu = ub[0] * cxv(i) + ub[1] * cyv(i) + ub[2] * czv(i);
-            f[(long long)q * N + n] = (float)(wv(i) * rls[l] * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu));
+            const int l = q >= 19, i = q - 19 * l;
+            const double cu =
+                signed_by(dir_of(i, 0), ub[0]) + signed_by(dir_of(i, 1), ub[1]) + signed_by(dir_of(i, 2), ub[2]);
+            f[(long long)q * N + n] = (float)(wv(i) * (l ? rB : rA) * (base + cu * (3.0 + 4.5 * cu)));
         }
-        if (lane == src) {
-            double pm[3] = {0, 0, 0};
-            for (int l = 0; l < 2; ++l) {
-                pm[0] += rls[l] * ub[0]; pm[1] += rls[l] * ub[1]; pm[2] += rls[l] * ub[2];
-            }
-            acc[0] -= pm[0]; acc[1] -= pm[1]; acc[2] -= pm[2];
-            acc[3] -= r[1] * pm[2] - r[2] * pm[1];
-            acc[4] -= r[2] * pm[0] - r[0] * pm[2];
-            acc[5] -= r[0] * pm[1] - r[1] * pm[0];
-            acc[6] -= rls[0];
-            acc[7] -= rls[1];
-        }
+        const double rt = rA + rB;
+        const double p[3] = {rt * ub[0], rt * ub[1], rt * ub[2]};
+        acc -= event_value(lane & 7, r, p, rA, rB);
     }
-    block_sum8<256>(acc, s_red, s_out);
-    if (threadIdx.x < 8) parts[blk * 8 + threadIdx.x] = s_out[threadIdx.x];
+    __syncthreads();  // s_any is cleared
+    if (lane < 8) s_red[(threadIdx.x >> 5) * 8 + lane] = acc;
+    if (lane == 0) {
+        s_cnt[threadIdx.x >> 5] = __popc(marked);
+        if (events) s_any = 1;
+    }
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        double s = 0.0;
+        if (s_any)
+            for (int w = 0; w < 256 / 32; ++w) s += s_red[w * 8 + threadIdx.x];
+        parts[blk * 8 + threadIdx.x] = s;
+    }
+    if (threadIdx.x == 0) {
+        int a = 0;
+        for (int w = 0; w < 256 / 32; ++w) a += s_cnt[w];
+        counts[blk] = a;
+    }
     __syncthreads();
 }
 
@@ -955,19 +1008,19 @@ __device__ __forceinline__ void finish_step(DevState* __restrict__ st, const int
 // A block of the cover/uncover pass, then, in the launch's last block, the
 // step's bookkeeping (finish_step).
 __device__ __forceinline__ void cover_then_finish(int blk, float* __restrict__ f, DevState* __restrict__ st,
-                                                  const uint8_t* __restrict__ masks, double* __restrict__ parts,
-                                                  const int* __restrict__ counts, const KParams& P)
+                                                  uint8_t* __restrict__ masks, double* __restrict__ parts,
+                                                  int* __restrict__ counts, const KParams& P)
 {
-    cover_block(blk, f, st, masks, parts, P);
+    cover_block(blk, f, st, masks, counts, parts, P);
     const int nb = (P.B * P.B * P.B + 255) / 256;
-    if (last_block(&st->cover_done, (unsigned)nb, threadIdx.x < 8))  // threads 0..7 wrote parts
+    if (last_block(&st->cover_done, (unsigned)nb, threadIdx.x < 8))  // threads 0..7 wrote parts and the count
         finish_step(st, counts, parts, nb, P);
     __syncthreads();
 }
 
 static __global__ void __launch_bounds__(256) k_cover(float* __restrict__ f, DevState* __restrict__ st,
-                                                      const uint8_t* __restrict__ masks, double* __restrict__ parts,
-                                                      const int* __restrict__ counts, KParams P)
+                                                      uint8_t* __restrict__ masks, double* __restrict__ parts,
+                                                      int* __restrict__ counts, KParams P)
 {
     cover_then_finish(blockIdx.x, f, st, masks, parts, counts, P);
 }
@@ -988,18 +1041,25 @@ __device__ __forceinline__ void finish_step(DevState* __restrict__ st, const int
         }
         return;
     }
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    long long cnt = 0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
+    // The record's values are loaded before the sums.
+    double led = 0.0, Fp = 0.0;
+    if (threadIdx.x < 2) led = st->ledger_bb[threadIdx.x];
+    if (threadIdx.x == 2) Fp = st->Fp;
+    const long long step = st->step;
+    const int cur = st->cur;
+    int box[6];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] += __ldcg(parts + b * 8 + k);
-        cnt += __ldcg(counts + b);
+    for (int a = 0; a < 3; ++a) {
+        box[a] = st->box0[a];
+        box[3 + a] = st->box_next[a];
     }
+    long long cnt = 0;
+    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) cnt += __ldcg(counts + b);
     // Particle nodes: an integer sum, the same in any order.
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, off);
     if ((threadIdx.x & 31) == 0) s_c[threadIdx.x >> 5] = cnt;
-    block_sum8<256>(acc, s_red, s_out);  // its barriers also publish s_c
+    sum_rows8(parts, nblocks, s_red, s_out);  // its barriers also publish s_c
     // Threads 0, 1, 2 form delta_A, delta_B and the counterforce at once
     // (FP64 divisions are slow here); thread 0 also the rest.
     if (threadIdx.x >= 3) return;
@@ -1008,11 +1068,13 @@ __device__ __forceinline__ void finish_step(DevState* __restrict__ st, const int
     const long long nf = P.N - solid;
     if (threadIdx.x < 2) {
         const int l = threadIdx.x;
-        st->delta[l] = (st->ledger_bb[l] + s_out[6 + l]) / (double)nf;
-        st->delta_f[l] = (float)st->delta[l];
+        const double delta = (led + s_out[6 + l]) / (double)nf;
+        st->delta[l] = delta;
+        st->delta_f[l] = (float)delta;
     } else {
-        st->fc = P.counterforce ? -st->Fp / (double)nf : 0.0;
-        st->fc_f = (float)st->fc;
+        const double fc = P.counterforce ? -Fp / (double)nf : 0.0;
+        st->fc = fc;
+        st->fc_f = (float)fc;
     }
     if (threadIdx.x != 0) return;
     for (int a = 0; a < 3; ++a) {
@@ -1020,11 +1082,14 @@ __device__ __forceinline__ void finish_step(DevState* __restrict__ st, const int
         st->Lpend[a] = s_out[3 + a];
     }
     st->nfluid = nf;
-    st->box_prev[0] = st->box0[0]; st->box_prev[1] = st->box0[1]; st->box_prev[2] = st->box0[2];
-    st->box0[0] = st->box_next[0]; st->box0[1] = st->box_next[1]; st->box0[2] = st->box_next[2];
-    st->cur = 1 - st->cur;
-    st->step += 1;
-    st->step_u32 = (uint32_t)st->step;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        st->box_prev[a] = box[a];
+        st->box0[a] = box[3 + a];
+    }
+    st->cur = 1 - cur;
+    st->step = step + 1;
+    st->step_u32 = (uint32_t)(step + 1);
 }
 
 static __global__ void __launch_bounds__(256) k_finish(DevState* __restrict__ st, const int* __restrict__ counts,
