@@ -829,6 +829,38 @@ __device__ __forceinline__ double event_value(int k, const double r[3], const do
     return k < 3 ? lin : (k < 6 ? cross : (k == 6 ? mA : mB));
 }
 
+// node_inside decided in float where the distance is clear of the surface by
+// more than the float's error can reach (coordinates good to 2^-23 of the
+// longest axis, squared distances within the box and its neighbours to that
+// times 4 (R + 4) and a few ulps), else in FP64: few nodes need the slow pipe.
+struct SphereTest {
+    float x[3], R2, margin;
+    __device__ __forceinline__ SphereTest(const double X[3], const KParams& P)
+    {
+        const float R = (float)P.R;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) x[a] = (float)X[a];
+        R2 = R * R;
+        margin = 1e-6f * ((R + 4.0f) * (float)max(P.lx, max(P.ly, P.lz)) + 8.0f * R2) + 1e-5f;
+    }
+    __device__ __forceinline__ bool inside(const int c[3], const double X[3], const KParams& P) const
+    {
+        const int L[3] = {P.lx, P.ly, P.lz};
+        float s = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            float r = (float)c[a] - x[a];
+            if (!P.wall[a]) {
+                if (r > 0.5f * L[a]) r -= L[a];
+                else if (r < -0.5f * L[a]) r += L[a];
+            }
+            s += r * r;
+        }
+        if (fabsf(s - R2) > margin) return s < R2;
+        return node_inside(c, X, P);
+    }
+};
+
 // (2) Particle nodes at the new position -> mask[1 - cur] and their count,
 // cover (new box) and uncover (old box) on the post-stream populations f;
 // per-block FP64 partials of impulse, angular impulse and mass ledger. Block
@@ -857,27 +889,28 @@ __device__ __forceinline__ void cover_block(int blk, float* __restrict__ f, cons
     const uint8_t* m_old = masks + (size_t)cur * B3;
     const int L[3] = {P.lx, P.ly, P.lz};
     const long long N = P.N;
+    const SphereTest sphere(X, P);
     if (threadIdx.x == 0) s_any = 0;
     bool now = false, covered = false, uncovered = false;
     int cc[3] = {0, 0, 0}, cu_[3] = {0, 0, 0};  // the covered / uncovered node of this thread
     if (t < B3) {
         const int d[3] = {t % B, (t / B) % B, t / (B * B)};
         const bool was = m_old[t] != 0;
-        now = box_node_inside(t, o_new, X, P);
-        masks[(size_t)(1 - cur) * B3 + t] = (uint8_t)now;
-        if (now) {
-            for (int a = 0; a < 3; ++a) {
-                cc[a] = o_new[a] + d[a];
-                if (!P.wall[a] && cc[a] >= L[a]) cc[a] -= L[a];
-            }
-            covered = !is_solid(cc[0], cc[1], cc[2], o_old, m_old, P);
+        now = true;
+        for (int a = 0; a < 3; ++a) {
+            cc[a] = o_new[a] + d[a];
+            if (P.wall[a]) now = now && cc[a] >= 0 && cc[a] < L[a];
+            else if (cc[a] >= L[a]) cc[a] -= L[a];
         }
+        now = now && sphere.inside(cc, X, P);
+        masks[(size_t)(1 - cur) * B3 + t] = (uint8_t)now;
+        if (now) covered = !is_solid(cc[0], cc[1], cc[2], o_old, m_old, P);
         if (was) {
             for (int a = 0; a < 3; ++a) {
                 cu_[a] = o_old[a] + d[a];
                 if (!P.wall[a] && cu_[a] >= L[a]) cu_[a] -= L[a];
             }
-            uncovered = !node_inside(cu_, X, P);
+            uncovered = !sphere.inside(cu_, X, P);
         }
     }
     const unsigned marked = __ballot_sync(0xffffffffu, now);
@@ -937,7 +970,7 @@ __device__ __forceinline__ void cover_block(int blk, float* __restrict__ f, cons
                 }
             }
             // a fluid neighbour that was fluid before as well
-            ok = ok && !is_solid(q[0], q[1], q[2], o_old, m_old, P) && !node_inside(q, X, P);
+            ok = ok && !is_solid(q[0], q[1], q[2], o_old, m_old, P) && !sphere.inside(q, X, P);
             if (ok) {
                 const long long m = q[0] + (long long)P.lx * (q[1] + (long long)P.ly * q[2]);
                 m0 = pop_sum(f, 0, m, N);
