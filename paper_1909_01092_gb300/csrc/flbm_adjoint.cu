@@ -100,26 +100,27 @@ using lg_t = Split;   // lambda g_l: 6 per node
 
 constexpr int kT = 256;  // threads per block
 
-// Sum of NV <= 8 doubles over the block by the tree of block_sum8 (so each
-// sum is the same), without reducing unused slots; s_out[0..NV) is the result.
-template <int NV>
-__device__ __forceinline__ void block_sum_n(const double v[NV], double* s_red, double* s_out)
+// Sum of four doubles over the block, as block_sum8 (a transposed butterfly
+// per warp: 2 + 1 + 1 + 1 + 1 FP64 additions a lane); s_out[0..3] is the result.
+__device__ __forceinline__ void block_sum4(const double v[4], double* s_red, double* s_out)
 {
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int lane = tid & 31, warp = tid >> 5;
     const int nwarp = (blockDim.x * blockDim.y + 31) >> 5;
+    const bool u4 = lane & 16, u3 = lane & 8;
+    double p[2];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double a = v[k];
+    for (int i = 0; i < 2; ++i)
+        p[i] = (u4 ? v[2 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, u4 ? v[i] : v[2 + i], 16);
+    double a = (u3 ? p[1] : p[0]) + __shfl_xor_sync(0xffffffffu, u3 ? p[0] : p[1], 8);
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
-        if (lane == 0) s_red[warp * 8 + k] = a;
-    }
+    for (int off = 4; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    if ((lane & 7) == 0) s_red[warp * 4 + (lane >> 4 & 1) * 2 + (lane >> 3 & 1)] = a;
     __syncthreads();
-    if (tid < NV) {
-        double a = 0.0;
-        for (int w = 0; w < nwarp; ++w) a += s_red[w * 8 + tid];
-        s_out[tid] = a;
+    if (tid < 4) {
+        double t = 0.0;
+        for (int w = 0; w < nwarp; ++w) t += s_red[w * 4 + tid];
+        s_out[tid] = t;
     }
     __syncthreads();
 }
@@ -614,7 +615,7 @@ __device__ __forceinline__ void adj_tile(int bx, int by, int bz, int tx, int ty,
                     wl[i] = wv(i) * dv;
                     wsum += wl[i];
                 }
-                acc[10 + l] += ax + (double)wsum;  // sum_i w_i lambda f*_li (mass correction)
+                acc[10 + l] = ax + (double)wsum;  // sum_i w_i lambda f*_li (mass correction)
                 float mm[10];
                 project10<float>(wl, mm);
                 for (int k = 0; k < 10; ++k) lm[l][k] = mm[k] / bnorm(k);
@@ -683,9 +684,9 @@ __device__ __forceinline__ void adj_tile(int bx, int by, int bz, int tx, int ty,
     } else if (tid < 9) {
         parts[tile * kNodeParts + tid] = 0.0;  // no link terms away from the particle
     }
-    double v4[kNodeParts - 8];
-    for (int k = 0; k < kNodeParts - 8; ++k) v4[k] = acc[8 + k];
-    block_sum_n<kNodeParts - 8>(v4, s_red, s_out);
+    static_assert(kNodeParts == 12, "the last four partials go through block_sum4");
+    const double v4[4] = {acc[8], acc[9], acc[10], acc[11]};
+    block_sum4(v4, s_red, s_out);
     if (tid < kNodeParts - 8) parts[tile * kNodeParts + 8 + tid] = s_out[tid];
 }
 

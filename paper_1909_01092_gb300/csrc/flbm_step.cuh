@@ -101,22 +101,18 @@ __device__ __forceinline__ float sqrt_newton(float x)
     return __fmaf_rn(__fmaf_rn(-s, s, x), __fmul_rn(0.5f, y), s);
 }
 
-// FP32 sums over the particle links of one node.
+// Sums over the particle links of one node. A link exchanges m c_i, m about
+// 2 w_i rho_tot; summed as they are in FP32, these cost the particle's force
+// more than the rounding of the populations does, although their uniform part
+// cancels around the sphere. So F holds what exceeds 2 w_i rho_l of each
+// component, and k = sum 36 w_i c_i, small whole numbers, the rest, which is
+// added in FP64. (The force acts along the lever c_i / 2 from the node: no
+// torque about it.)
 struct LinkSums {
-    float F[3] = {0.0f, 0.0f, 0.0f};    // force on the particle
-    float T[3] = {0.0f, 0.0f, 0.0f};    // torque about the node (lever c_i / 2)
+    float F[3] = {0.0f, 0.0f, 0.0f};    // force on the particle beyond 2 w_i rho_tot c_i
+    int k[3] = {0, 0, 0};
     float led[2] = {0.0f, 0.0f};        // mass put in by the moving link rule
 };
-
-// Adds the force m c_i acting at the link midpoint x + c_i / 2.
-__device__ __forceinline__ void link_add(LinkSums& s, float m, int cx, int cy, int cz)
-{
-    const float fr[3] = {m * cx, m * cy, m * cz};
-    s.F[0] += fr[0]; s.F[1] += fr[1]; s.F[2] += fr[2];
-    s.T[0] += 0.5f * (cy * fr[2] - cz * fr[1]);
-    s.T[1] += 0.5f * (cz * fr[0] - cx * fr[2]);
-    s.T[2] += 0.5f * (cx * fr[1] - cy * fr[0]);
-}
 
 // Densities and momenta of both components from their populations.
 __device__ __forceinline__ void moments(const Pair f[19], Pair& rho, Pair j[3])
@@ -360,7 +356,7 @@ __device__ __forceinline__ void load_force(const In& in, NodeState<TAU1>& s)
 
 // Collision and push-streaming of one fluid node (Eq. (lbe)) from its loaded
 // state. With PARTICLE, solid_nb marks the directions whose neighbour is a
-// particle node; their links take the moving rule and feed acc = (F[3], T[3],
+// particle node; their links take the moving rule and give acc = (F[3], T[3],
 // ledger[2]). TAU1: every relaxation time is 1, so the post-collision modes
 // depend on the input only through rho_l and j_l, and the ghost modes carry
 // noise only. The outputs are pushed to fout, population (l, i) of node m at
@@ -456,9 +452,9 @@ __device__ __forceinline__ void collide_push(int x, int y, int z, uint32_t n, co
         from_modes(k, fo);
     }
 
-    // Particle links of this node: FP32 sums of force, torque about the node
-    // (lever c_i / 2) and mass ledger, moved into the FP64 accumulators once
-    // per node; relative position of the node to the particle centre in FP64.
+    // Particle links of this node: sums of force and mass ledger, moved into
+    // the FP64 accumulators once per node; relative position of the node to
+    // the particle centre in FP64.
     LinkSums lk;
     double rn[3] = {0.0, 0.0, 0.0};
     float rnf[3] = {0.0f, 0.0f, 0.0f};
@@ -492,9 +488,12 @@ __device__ __forceinline__ void collide_push(int x, int y, int z, uint32_t n, co
             const Pair back = sub(fo[i], corr);
             fout[back_idx] = back.x;
             foutB[back_idx] = back.y;
-            const Pair pn = in.psi(i);
-            const Pair ex = add(fo[i], back);
-            link_add(lk, (ex.x + ex.y) + P.G * wv(i) * (rho.x * pn.x + rho.y * pn.y), cx, cy, cz);
+            const Pair pn = in.psi(i), mw = splat(-wv(i));
+            const Pair ex = add(mad(mw, rho, fo[i]), mad(mw, rho, back));
+            const float m = (ex.x + ex.y) + P.G * wv(i) * (rho.x * pn.x + rho.y * pn.y);
+            lk.F[0] += m * cx; lk.F[1] += m * cy; lk.F[2] += m * cz;
+            const int w36 = i <= 6 ? 2 : 1;
+            lk.k[0] += w36 * cx; lk.k[1] += w36 * cy; lk.k[2] += w36 * cz;
             lk.led[0] += corr.x;
             lk.led[1] += corr.y;
             continue;
@@ -510,13 +509,16 @@ __device__ __forceinline__ void collide_push(int x, int y, int z, uint32_t n, co
         }
     }
     if (PARTICLE && solid_nb) {
-        const double F[3] = {lk.F[0], lk.F[1], lk.F[2]};
-        acc[0] += F[0]; acc[1] += F[1]; acc[2] += F[2];
-        acc[3] += rn[1] * F[2] - rn[2] * F[1] + lk.T[0];
-        acc[4] += rn[2] * F[0] - rn[0] * F[2] + lk.T[1];
-        acc[5] += rn[0] * F[1] - rn[1] * F[0] + lk.T[2];
-        acc[6] += lk.led[0];
-        acc[7] += lk.led[1];
+        const double base = 2.0 * (double)wv(7) * ((double)rho.x + (double)rho.y);
+        double F[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) F[a] = (double)lk.F[a] + base * (double)lk.k[a];
+        acc[0] = F[0]; acc[1] = F[1]; acc[2] = F[2];
+        acc[3] = rn[1] * F[2] - rn[2] * F[1];
+        acc[4] = rn[2] * F[0] - rn[0] * F[2];
+        acc[5] = rn[0] * F[1] - rn[1] * F[0];
+        acc[6] = lk.led[0];
+        acc[7] = lk.led[1];
     }
 }
 
