@@ -466,6 +466,15 @@ static __global__ void __launch_bounds__(kT) ka_cover_mean(lam_t* __restrict__ l
 // node's b_l and the local part of a_l into lam0, lambda g_l into lg, and
 // per-tile partials (link terms of lambda X, V, Omega; dJ/dG; lambda delta).
 // ---------------------------------------------------------------------------
+// (lambda F + lambda T x d) . c_i at the midpoint d of the link along c_i: the
+// adjoint of the momentum the link gives the particle.
+__device__ __forceinline__ float link_kappa(int cx, int cy, int cz, const float rnf[3], const float* lF, const float* lT)
+{
+    const float d[3] = {rnf[0] + 0.5f * cx, rnf[1] + 0.5f * cy, rnf[2] + 0.5f * cz};
+    return cx * (lF[0] + lT[1] * d[2] - lT[2] * d[1]) + cy * (lF[1] + lT[2] * d[0] - lT[0] * d[2]) +
+           cz * (lF[2] + lT[0] * d[1] - lT[1] * d[0]);
+}
+
 // Thread (tx, ty) of tile (bx, by, bz); every thread of the block calls it.
 // PARTICLE: the tile is near the particle (links, reaction); else it has none.
 template <bool PARTICLE>
@@ -567,44 +576,7 @@ __device__ __forceinline__ void adj_tile(int bx, int by, int bz, int tx, int ty,
                     if ((wall_nb | solid_nb) >> i & 1u) {
                         // bounce-back reads (x, -c_i): a - c_i . b, so dv = -2 c_i . b (float)
                         dv = -2.0f * (cx * bs[0].hi + cy * bs[1].hi + cz * bs[2].hi);
-                        if (PARTICLE && (solid_nb >> i & 1u)) {
-                            // The large adjoint parts (a_l, b_l and the ledger's) in double-float,
-                            // the forward quantities in float.
-                            df cb;
-                            if (cx) cb += cx > 0 ? df(bs[0].hi, bs[0].lo) : -df(bs[0].hi, bs[0].lo);
-                            if (cy) cb += cy > 0 ? df(bs[1].hi, bs[1].lo) : -df(bs[1].hi, bs[1].lo);
-                            if (cz) cb += cz > 0 ? df(bs[2].hi, bs[2].lo) : -df(bs[2].hi, bs[2].lo);
-                            const float d[3] = {rnf[0] + 0.5f * cx, rnf[1] + 0.5f * cy, rnf[2] + 0.5f * cz};
-                            const float kap = cx * (lF[0] + lT[1] * d[2] - lT[2] * d[1]) +
-                                              cy * (lF[1] + lT[2] * d[0] - lT[0] * d[2]) +
-                                              cz * (lF[2] + lT[0] * d[1] - lT[1] * d[0]);
-                            const float* V = s0->Vf;
-                            const float* Om = s0->Omf;
-                            const float ubc = (V[0] + Om[1] * d[2] - Om[2] * d[1]) * cx +
-                                              (V[1] + Om[2] * d[0] - Om[0] * d[2]) * cy +
-                                              (V[2] + Om[0] * d[1] - Om[1] * d[0]) * cz;
-                            const df lcorr = (cb - df(as.hi, as.lo)) + (lled[l] + (-kap));
-                            const float w6 = 6.0f * wv(i);
-                            lrx[l] += lcorr * (w6 * ubc);
-                            const df lub = lcorr * (w6 * rho[l]);  // lambda (u_b . c_i)
-                            // With lb = lub c_i: partials 3..5 += lb, 6..8 += d x lb,
-                            // 0..2 -= lb x Omega (the float sums of coefficients exact).
-                            if (cx) lk[3] += cx > 0 ? lub : -lub;
-                            if (cy) lk[4] += cy > 0 ? lub : -lub;
-                            if (cz) lk[5] += cz > 0 ? lub : -lub;
-                            lk[6] += lub * two_sum(d[1] * cz, -d[2] * cy);
-                            lk[7] += lub * two_sum(d[2] * cx, -d[0] * cz);
-                            lk[8] += lub * two_sum(d[0] * cy, -d[1] * cx);
-                            lk[0] += lub * two_sum(cz * Om[1], -cy * Om[2]);
-                            lk[1] += lub * two_sum(cx * Om[2], -cz * Om[0]);
-                            lk[2] += lub * two_sum(cy * Om[0], -cx * Om[1]);
-                            // lever of the exchanged momentum (2 f* - corr) c_i (small: float)
-                            const float dp = 2.0f * fo[l][i] - w6 * rho[l] * ubc;
-                            lk[0] = lk[0] + (-dp * (cy * lT[2] - cz * lT[1]));
-                            lk[1] = lk[1] + (-dp * (cz * lT[0] - cx * lT[2]));
-                            lk[2] = lk[2] + (-dp * (cx * lT[1] - cy * lT[0]));
-                            dv += 2.0f * kap;
-                        }
+                        if (PARTICLE && (solid_nb >> i & 1u)) dv += 2.0f * link_kappa(cx, cy, cz, rnf, lF, lT);
                     } else {
                         const uint32_t q = qidx[i];
                         dv = sdiff(lam1[(size_t)l * N + q], as);
@@ -616,22 +588,61 @@ __device__ __forceinline__ void adj_tile(int bx, int by, int bz, int tx, int ty,
                     wsum += wl[i];
                 }
                 acc[10 + l] = ax + (double)wsum;  // sum_i w_i lambda f*_li (mass correction)
+                // The links, one copy of their code for all directions: unrolled
+                // like the gathers it filled the instruction cache many times over.
+                if (PARTICLE) {
+#pragma unroll 1
+                    for (uint32_t left = solid_nb; left; left &= left - 1u) {
+                        const int i = __ffs(left) - 1;
+                        const int cx = dir_of(i, 0), cy = dir_of(i, 1), cz = dir_of(i, 2);
+                        // The large adjoint parts (a_l, b_l and the ledger's) in double-float,
+                        // the forward quantities in float.
+                        df cb;
+                        if (cx) cb += cx > 0 ? df(bs[0].hi, bs[0].lo) : -df(bs[0].hi, bs[0].lo);
+                        if (cy) cb += cy > 0 ? df(bs[1].hi, bs[1].lo) : -df(bs[1].hi, bs[1].lo);
+                        if (cz) cb += cz > 0 ? df(bs[2].hi, bs[2].lo) : -df(bs[2].hi, bs[2].lo);
+                        const float d[3] = {rnf[0] + 0.5f * cx, rnf[1] + 0.5f * cy, rnf[2] + 0.5f * cz};
+                        const float kap = link_kappa(cx, cy, cz, rnf, lF, lT);
+                        const float* V = s0->Vf;
+                        const float* Om = s0->Omf;
+                        const float ubc = (V[0] + Om[1] * d[2] - Om[2] * d[1]) * cx +
+                                          (V[1] + Om[2] * d[0] - Om[0] * d[2]) * cy +
+                                          (V[2] + Om[0] * d[1] - Om[1] * d[0]) * cz;
+                        const df lcorr = (cb - df(as.hi, as.lo)) + (lled[l] + (-kap));
+                        const float w6 = 6.0f * wv(i);
+                        lrx[l] += lcorr * (w6 * ubc);
+                        const df lub = lcorr * (w6 * rho[l]);  // lambda (u_b . c_i)
+                        // With lb = lub c_i: partials 3..5 += lb, 6..8 += d x lb,
+                        // 0..2 -= lb x Omega (the float sums of coefficients exact).
+                        if (cx) lk[3] += cx > 0 ? lub : -lub;
+                        if (cy) lk[4] += cy > 0 ? lub : -lub;
+                        if (cz) lk[5] += cz > 0 ? lub : -lub;
+                        lk[6] += lub * two_sum(d[1] * cz, -d[2] * cy);
+                        lk[7] += lub * two_sum(d[2] * cx, -d[0] * cz);
+                        lk[8] += lub * two_sum(d[0] * cy, -d[1] * cx);
+                        lk[0] += lub * two_sum(cz * Om[1], -cy * Om[2]);
+                        lk[1] += lub * two_sum(cx * Om[2], -cz * Om[0]);
+                        lk[2] += lub * two_sum(cy * Om[0], -cx * Om[1]);
+                        // lever of the exchanged momentum (2 f* - corr) c_i (small: float)
+                        const float dp = 2.0f * fo[l][i] - w6 * rho[l] * ubc;
+                        lk[0] = lk[0] + (-dp * (cy * lT[2] - cz * lT[1]));
+                        lk[1] = lk[1] + (-dp * (cz * lT[0] - cx * lT[2]));
+                        lk[2] = lk[2] + (-dp * (cx * lT[1] - cy * lT[0]));
+                    }
+                }
                 float mm[10];
                 project10<float>(wl, mm);
                 for (int k = 0; k < 10; ++k) lm[l][k] = mm[k] / bnorm(k);
             }
             // Shan-Chen reaction on the particle: F += G w_i (rhoA psiB(q) + rhoB psiA(q)) c_i.
             if (PARTICLE && solid_nb) {
-#pragma unroll
-                for (int i = 1; i < 19; ++i) {
-                    if (!(solid_nb >> i & 1u)) continue;
-                    const int cx = cxv(i), cy = cyv(i), cz = czv(i);
+#pragma unroll 1
+                for (uint32_t left = solid_nb; left; left &= left - 1u) {
+                    const int i = __ffs(left) - 1;
+                    const int cx = dir_of(i, 0), cy = dir_of(i, 1), cz = dir_of(i, 2);
                     const int off = cx + sy * cy + sz * cz;
                     const float pa = pA[off], pb = pB[off];
-                    const float d[3] = {rnf[0] + 0.5f * cx, rnf[1] + 0.5f * cy, rnf[2] + 0.5f * cz};
-                    const float kap = cx * (lF[0] + lT[1] * d[2] - lT[2] * d[1]) +
-                                      cy * (lF[1] + lT[2] * d[0] - lT[0] * d[2]) +
-                                      cz * (lF[2] + lT[0] * d[1] - lT[1] * d[0]);
+                    const float kap = link_kappa(cx, cy, cz, rnf, lF, lT);
                     const float w = wv(i);
                     const float t = rho[0] * pb + rho[1] * pa;
                     lk[9] += two_prod(kap * w, t);

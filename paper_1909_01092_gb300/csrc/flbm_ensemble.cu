@@ -9,9 +9,9 @@
 // stages the descriptor of its current replica (kernel parameters and device
 // pointers) in shared memory and runs the same device bodies as the
 // single-simulation kernels, so each replica computes exactly what
-// flbm_create/flbm_step would. With one block per item, the bulk collide
-// instead takes the descriptors of up to kChunkReps replicas as a kernel
-// parameter (kb_bulk_rep). The step sequence (densities; density shell;
+// flbm_create/flbm_step would. The bulk collide instead takes the descriptors
+// of up to kChunkReps replicas as a kernel parameter (kb_bulk_rep), unless that
+// takes many launches a step in a persistent configuration. The step sequence (densities; density shell;
 // collide-stream of the bulk tiles; on a side stream meanwhile the virtual
 // layer and the near tiles, whose launch ends with each replica's particle
 // update; next-position masks and cover/uncover ending with each replica's
@@ -91,12 +91,17 @@ __device__ __forceinline__ TileCoord tile_of(const Item& it, const KParams& P)
         const KParams& P = sR.P;
 #define FLBM_END_ITEMS }
 
-static __global__ void __launch_bounds__(256) kb_density(const RepDesc* __restrict__ reps,
+// Persistent blocks (PERSIST) keep a node's 38 loads in flight, in 64
+// registers: there are only a few of them. One block per item does better with
+// 32 registers and eight blocks per SM, among which the descriptors' staging
+// hides (128 replicas: 1.04 ms a step against 1.19 ms).
+template <bool PERSIST>
+static __global__ void __launch_bounds__(256, PERSIST ? 4 : 8) kb_density(const RepDesc* __restrict__ reps,
                                                          const Item* __restrict__ items, int nitems, int par)
 {
     FLBM_FOR_ITEMS
     const TileCoord c = tile_of(it, P);
-    density_node(c.bx * P.tx + c.tx, c.by * P.ty + c.ty, c.bz, sR.f[par], sR.psi, sR.st, sR.masks, P);
+    density_node<PERSIST>(c.bx * P.tx + c.tx, c.by * P.ty + c.ty, c.bz, sR.f[par], sR.psi, sR.st, sR.masks, P);
     FLBM_END_ITEMS
 }
 
@@ -222,9 +227,10 @@ struct flbm_ens {
     Item* d_items = nullptr;
     size_t items_cap = 0;
     long long off[W_COUNT + 1] = {};  // work list k = d_items[off[k] .. off[k+1])
-    // Bulk collide launches of one block per tile (ctas_per_sm 0), per
-    // variant: replicas of similar tile counts grouped, kChunkReps at most
-    // per launch.
+    // Bulk collide launches of one block per tile, per variant: replicas of
+    // similar tile counts grouped, kChunkReps at most per launch; in use with
+    // ctas_per_sm 0, and otherwise while they are few.
+    bool bulk_by_reps = false;
     struct RepLaunch {
         RepChunk c;
         int n = 0;
@@ -342,6 +348,14 @@ int apply_config(flbm_ens* e)
             for (int r : g) ch.back().c.r[ch.back().n++] = e->rd[r];
         }
     }
+    // The descriptors in the constant bank instead of shared memory leave the
+    // update its registers: 15 channels of 60x60x120 take 480 us a step through
+    // the lists' kernel; their step falls from 1.06 to 0.91 ms with these. Persistent
+    // configurations keep the lists only where the replicas' sizes would ask
+    // for many launches.
+    size_t reps = 0;
+    for (int k = 0; k < 4; ++k) reps += e->rep_launches[k].size();
+    e->bulk_by_reps = e->cfg.ctas_per_sm == 0 || reps <= 4;
     if (items.size() > (size_t)0x7fffffff) return efail(e, FLBM_E_INVAL, "too many work items");
     if (items.size() > e->items_cap) {
         cudaFree(e->d_items);
@@ -481,7 +495,9 @@ int launch_bulk_reps(flbm_ens* e, int par)
 int ens_step(flbm_ens* e)
 {
     const int par = e->cur;
-    if (int rc = launch_list(e, W_DENSITY, kb_density, "kb_density", par)) return rc;
+    if (int rc = e->cfg.ctas_per_sm > 0 ? launch_list(e, W_DENSITY, kb_density<true>, "kb_density", par)
+                                        : launch_list(e, W_DENSITY, kb_density<false>, "kb_density", par))
+        return rc;
     // The particles' share of the step runs on the side stream: the virtual
     // layers once the densities are in, the near tiles once the shells are
     // in too. The shells and the bulk tiles, which read neither, run on the
@@ -504,7 +520,7 @@ int ens_step(flbm_ens* e)
         if (int rc = launch_on(e, e->side, W_NEAR + 3, kb_near<true, true>, "kb_near", par)) return rc;
         ECK(e, cudaEventRecord(e->join_ev, e->side));
     }
-    if (e->cfg.ctas_per_sm == 0) {
+    if (e->bulk_by_reps) {
         if (int rc = launch_bulk_reps(e, par)) return rc;
     } else {
         if (int rc = launch_list(e, W_BULK + 0, kb_bulk<false, false>, "kb_bulk", par)) return rc;

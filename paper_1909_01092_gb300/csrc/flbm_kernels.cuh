@@ -46,6 +46,8 @@ static __global__ void __launch_bounds__(kThreads) k_init(float* __restrict__ f,
 // ---------------------------------------------------------------------------
 // Densities of fluid nodes into the psi interior; 0 on particle nodes.
 // ---------------------------------------------------------------------------
+// TOGETHER: the loads first, all in flight, then the sums (the same order).
+template <bool TOGETHER = false>
 __device__ __forceinline__ void density_node(int x, int y, int z, const float* __restrict__ f, float* __restrict__ psi,
                                              const DevState* __restrict__ st, const uint8_t* __restrict__ masks,
                                              const KParams& P)
@@ -58,7 +60,23 @@ __device__ __forceinline__ void density_node(int x, int y, int z, const float* _
         solid = is_solid(x, y, z, o, masks + (size_t)st->cur * P.B * P.B * P.B, P);
     }
     float ra = 0.0f, rb = 0.0f;
-    if (!solid) {
+    if (TOGETHER) {
+        float va[19], vb[19];
+        const float *pa = f + n, *pb = f + 19 * P.N + n;
+        const long long N = P.N;
+#pragma unroll
+        for (int i = 0; i < 19; ++i, pa += N, pb += N) {
+            va[i] = __ldg(pa);
+            vb[i] = __ldg(pb);
+        }
+        if (!solid) {
+#pragma unroll
+            for (int i = 0; i < 19; ++i) {
+                ra += va[i];
+                rb += vb[i];
+            }
+        }
+    } else if (!solid) {
 #pragma unroll
         for (int i = 0; i < 19; ++i) {
             ra += f[(long long)i * P.N + n];
