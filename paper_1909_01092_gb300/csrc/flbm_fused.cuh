@@ -192,23 +192,28 @@ struct DensitySink {
 #pragma unroll
         for (int l = 0; l < 2; ++l) own[l][0] = own[l][1] = own[l][2] = 0.0f;
     }
+    // The own column's share of population i of component l.
+    __host__ __device__ __forceinline__ void put_own(int l, int i, float v, bool bounced)
+    {
+        if (i == 0 || bounced) own[l][1] += v;
+        else if (i == 5) own[l][2] += v;
+        else if (i == 6) own[l][0] += v;
+    }
     __host__ __device__ __forceinline__ void put(int l, int i, float v, bool bounced)
     {
-        if (i == 0) {
-            own[l][1] += v;
-            return;
-        }
-        if (bounced) own[l][1] += v;
-        if (i == 5) {
-            if (!bounced) own[l][2] += v;
-        } else if (i == 6) {
-            if (!bounced) own[l][0] += v;
-        } else {
-            // A bounced value is stored too: its target lies across the wall,
-            // where no node and no ring position gathers it.
-            xch[2 * (xch_slot(i) * size + pos) + l] = v;
-        }
+        put_own(l, i, v, bounced);
+        // A bounced value is stored too: its target lies across the wall,
+        // where no node and no ring position gathers it.
+        if (leaves(i)) xch[2 * (xch_slot(i) * size + pos) + l] = v;
     }
+    // Both components: one 8-byte store.
+    __device__ __forceinline__ void put(int i, Pair v, bool bounced)
+    {
+        put_own(0, i, v.x, bounced);
+        put_own(1, i, v.y, bounced);
+        if (leaves(i)) reinterpret_cast<float2*>(xch)[xch_slot(i) * size + pos] = make_float2(v.x, v.y);
+    }
+    static __host__ __device__ constexpr bool leaves(int i) { return i != 0 && i != 5 && i != 6; }
 };
 
 // Values pushed into the column at exchange position p from the tile's
@@ -314,7 +319,12 @@ struct RingDuty {
     }
 };
 
-constexpr int kFusedBlocks = 4;  // resident blocks per SM of the fused collide
+// Resident blocks per SM of the fused collide. The packed update holds both
+// components' 38 pushed values at once, beside the sums of the own column: it
+// needs 128 registers. At four blocks (64) its spills go through to L2 and a
+// step of 128x128x512 with noise takes 1420 us, at three (80) 920 us, at two
+// 955 us; 60x60x900 takes 839 / 528 / 419 us, 64x64x128 152 / 119 / 108 us.
+constexpr int kFusedBlocks = 2;
 
 template <bool NOISE, bool TAU1>
 static __global__ void __launch_bounds__(kThreadsStep, kFusedBlocks)

@@ -237,13 +237,13 @@ struct PushFrame {
 };
 
 // Receiver of the pushed populations for callers that also want the next
-// step's densities (the fused bulk collide); put(l, i, v, bounced) sees every
-// population v = f*_li the node pushes outside the particle, bounced = true
+// step's densities (the fused bulk collide); put(i, v, bounced) sees every
+// pair of populations v = f*_li the node pushes outside the particle, bounced = true
 // when a wall sent it back into the node itself. The default receiver does
 // nothing and compiles away.
 struct NoSink {
     static constexpr bool active = false;
-    __device__ __forceinline__ void put(int, int, float, bool) {}
+    __device__ __forceinline__ void put(int, Pair, bool) {}
 };
 
 // sqrt(1 / b_k): the noise amplitude of normalised mode k >= 4 per
@@ -503,10 +503,7 @@ __device__ __forceinline__ void collide_push(int x, int y, int z, uint32_t n, co
         const int pair = i == 0 ? 0 : (i & 1) ? i : i - 1;
         *at(fout + P.dirN[pair], to) = fo[i].x;
         *at(fout + P.dirN[19 + pair], to) = fo[i].y;
-        if constexpr (Sink::active) {
-            sink->put(0, i, fo[i].x, wall);
-            sink->put(1, i, fo[i].y, wall);
-        }
+        if constexpr (Sink::active) sink->put(i, fo[i], wall);
     }
     if (PARTICLE && solid_nb) {
         const double base = 2.0 * (double)wv(7) * ((double)rho.x + (double)rho.y);
