@@ -254,8 +254,8 @@ int flbm_restore(flbm_t* h, const char* path);
 int flbm_use_graphs(flbm_t* h, int enable);
 
 /* Bulk collide-stream with its inputs staged by the Tensor Memory Accelerator
- * (same node update, Section 2, Eq. (lbe)): a persistent grid copies each
- * tile's 38 x 256 populations and its padded density stencil into shared
+ * (same node update, Section 2, Eq. (lbe)): each block copies its
+ * tiles' 38 x 256 populations and padded density stencil into shared
  * memory with tensor copies, double-buffered, while the previous tile is
  * computed. Available when the lattice allows it (lx % 4 == 0 and
  * lx >= 32); off by default, since the kernel that reads global memory

@@ -128,7 +128,7 @@ void setup_tma(flbm_sim* h)
             cudaSuccess ||
         per_sm < 1)
         return;
-    h->tma_grid = (int)std::min<long long>(h->ntiles, (long long)sms * per_sm);
+    h->tma_grid = (int)std::min<long long>(h->ntiles, (long long)sms * per_sm * kTmaWaves);
     h->tma_ok = true;  // available; flbm_use_tma switches it on
 }
 
@@ -286,7 +286,7 @@ int launch_step(flbm_sim* h, cudaEvent_t* ev = nullptr)
 }
 
 // Planes per block of the fused collide by default: enough chunks for about
-// two waves of resident blocks (4 per SM) over the lattice's tiles.
+// two waves of resident blocks over the lattice's tiles.
 int auto_chunk(const KParams& k)
 {
     int dev = 0, sms = 148;

@@ -63,7 +63,7 @@ struct flbm_sim {
     dim3 grid, block;
     // Bulk collide with TMA-staged inputs (k_collide_bulk_tma): tensor maps of
     // the two population copies and of the padded densities; tma_ok when the
-    // lattice allows it, tma when it is in use; persistent grid size.
+    // lattice allows it, tma when it is in use; its grid size.
     CUtensorMap tm_f[2];
     CUtensorMap tm_psi[2];
     bool tma_ok = false;

@@ -3,13 +3,14 @@
 //
 // The same node update as k_collide_bulk (collide_core), for lattices whose
 // rows are a multiple of 16 bytes (lx % 4 == 0) and whose tiles are 32 x 8
-// nodes of one z-plane. A persistent grid (two blocks per SM) walks the
-// tiles that are not next to the particle. For each tile one thread issues
+// nodes of one z-plane. Each block (two per SM resident, kTmaWaves times as
+// many launched) walks a share of the tiles that are not next to the particle. For each tile one thread issues
 // two tensor copies into a shared-memory stage: the 38 populations of the
 // tile's 256 nodes (38 x 8 x 32 floats) and the padded densities the
 // Shan-Chen stencil reads (2 components x 3 planes x 10 rows x 36 columns).
 // Two stages alternate: while the block works on one tile, the copies of its
-// next tile are in flight, so the HBM reads no longer wait on the warps. The
+// next tile are in flight, and a stage is refilled as soon as its tile's
+// moments and stencil sums are in registers, before the update. The
 // stores of the streamed populations go straight to global memory as before.
 //
 // Every wait on a stage's mbarrier is bounded: the waits for a tile's inputs
@@ -127,6 +128,14 @@ __device__ __forceinline__ void tile_coords(long long t, const KParams& P, int& 
     bz = (int)(r / P.gy);
 }
 
+// Blocks launched per resident one. With one each, the tiles are dealt out for
+// good, and the launch ends with its slowest SM: the noise-free update waits
+// for memory, which some SMs reach faster, and blocks beside the near launch
+// start late. Steps with 1 / 2 / 4 / 8: 128x128x512 noise-free 917 / 778 /
+// 745 / 700 us, with noise 807 / 793 / 781 / 787 us; 100x100x200 noise-free
+// 279 / 257 / 231 / 220 us, 64x64x128 with noise 101 / 95 / 94 / 98 us.
+constexpr int kTmaWaves = 8;
+
 template <bool NOISE, bool TAU1>
 static __global__ void __launch_bounds__(kThreadsStep, 2)
     k_collide_bulk_tma(const __grid_constant__ CUtensorMap tm_f, const __grid_constant__ CUtensorMap tm_psi,
@@ -198,14 +207,18 @@ static __global__ void __launch_bounds__(kThreadsStep, 2)
         int bx, by, bz;
         tile_coords(t, P, bx, by, bz);
         const int x = bx * kTmaTX + tx, y = by * kTmaTY + ty;
-        if (x < P.lx && y < P.ly) {
-            const uint32_t n = (uint32_t)x + (uint32_t)P.lx * ((uint32_t)y + (uint32_t)P.ly * (uint32_t)bz);
-            const StagedInputs in(reinterpret_cast<const float*>(smem + s * kTmaStageBytes), tx, ty);
-            collide_core<NOISE, false, TAU1>(x, y, bz, n, in, fout, st, P, 0u, nullptr);
+        const uint32_t n = (uint32_t)x + (uint32_t)P.lx * ((uint32_t)y + (uint32_t)P.ly * (uint32_t)bz);
+        const bool node = x < P.lx && y < P.ly;
+        const StagedInputs in(reinterpret_cast<const float*>(smem + s * kTmaStageBytes), tx, ty);
+        NodeState<TAU1> state;
+        if (node) {
+            load_modes(in, P, state);
+            load_force(in, state);
         }
         __syncthreads();  // every thread is done with stage s
         const long long t2 = next(tn);
         if (leader && t2 < ntiles) issue(t2, s);
+        if (node) collide_push<NOISE, false, TAU1>(x, y, bz, n, in, state, fout, st, P, 0u, nullptr);
         t = tn;
         tn = t2;
     }
