@@ -17,6 +17,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #include "flbm_pair.h"
 
@@ -60,7 +61,7 @@ __host__ __device__ constexpr float bnorm(int k)
 
 // Forward mode transform m_k = sum_i e_k(c_i) f_i of the D3Q19 MRT basis
 // (density, momentum, 6 stress, 9 ghost modes), evaluated with opposite-pair
-// sums (even modes) and differences (odd modes); T = double in the observables.
+// sums (even modes) and differences (odd modes), in FP64 for the observables.
 template <class T>
 __host__ __device__ __forceinline__ void to_modes_t(const T f[19], T m[19])
 {
@@ -97,38 +98,37 @@ __host__ __device__ __forceinline__ void to_modes_t(const T f[19], T m[19])
     m[18] = -s2 + s3 + sxy - sxz;
 }
 
-__host__ __device__ __forceinline__ void to_modes(const float f[19], float m[19]) { to_modes_t<float>(f, m); }
-
-// The same transform in packed arithmetic (both components at once), every
-// operation written out.
-__device__ __forceinline__ void to_modes(const Pair f[19], Pair m[19])
+// The same transform with every operation written out; T = Pair in the step
+// (both components at once).
+template <class T>
+__host__ __device__ __forceinline__ void to_modes(const T f[19], T m[19])
 {
-    const Pair two = splat(2.0f), mtwo = splat(-2.0f);
-    const Pair s1 = add(f[1], f[2]), d1 = sub(f[1], f[2]);
-    const Pair s2 = add(f[3], f[4]), d2 = sub(f[3], f[4]);
-    const Pair s3 = add(f[5], f[6]), d3 = sub(f[5], f[6]);
-    const Pair s7 = add(f[7], f[8]), d7 = sub(f[7], f[8]);
-    const Pair s9 = add(f[9], f[10]), d9 = sub(f[9], f[10]);
-    const Pair s11 = add(f[11], f[12]), d11 = sub(f[11], f[12]);
-    const Pair s13 = add(f[13], f[14]), d13 = sub(f[13], f[14]);
-    const Pair s15 = add(f[15], f[16]), d15 = sub(f[15], f[16]);
-    const Pair s17 = add(f[17], f[18]), d17 = sub(f[17], f[18]);
-    const Pair s23 = add(s2, s3), sax = add(s1, s23);
-    const Pair sxy = add(s7, s9), sxz = add(s11, s13), syz = add(s15, s17);
-    const Pair sxx = add(sxy, sxz), sdg = add(sxx, syz);
+    const T two = lit<T>(2.0f), mtwo = lit<T>(-2.0f);
+    const T s1 = add(f[1], f[2]), d1 = sub(f[1], f[2]);
+    const T s2 = add(f[3], f[4]), d2 = sub(f[3], f[4]);
+    const T s3 = add(f[5], f[6]), d3 = sub(f[5], f[6]);
+    const T s7 = add(f[7], f[8]), d7 = sub(f[7], f[8]);
+    const T s9 = add(f[9], f[10]), d9 = sub(f[9], f[10]);
+    const T s11 = add(f[11], f[12]), d11 = sub(f[11], f[12]);
+    const T s13 = add(f[13], f[14]), d13 = sub(f[13], f[14]);
+    const T s15 = add(f[15], f[16]), d15 = sub(f[15], f[16]);
+    const T s17 = add(f[17], f[18]), d17 = sub(f[17], f[18]);
+    const T s23 = add(s2, s3), sax = add(s1, s23);
+    const T sxy = add(s7, s9), sxz = add(s11, s13), syz = add(s15, s17);
+    const T sxx = add(sxy, sxz), sdg = add(sxx, syz);
     // the odd sums of the diagonal directions, per axis
-    const Pair ax = add(add(d7, d9), add(d11, d13));
-    const Pair ay = add(sub(d7, d9), add(d15, d17));
-    const Pair az = add(sub(d11, d13), sub(d15, d17));
+    const T ax = add(add(d7, d9), add(d11, d13));
+    const T ay = add(sub(d7, d9), add(d15, d17));
+    const T az = add(sub(d11, d13), sub(d15, d17));
     m[0] = add(f[0], add(sax, sdg));
     m[1] = add(d1, ax);
     m[2] = add(d2, ay);
     m[3] = add(d3, az);
     m[4] = sub(sdg, f[0]);
-    const Pair sq = mad(mtwo, syz, sxx);  // s_xy + s_xz - 2 s_yz
-    const Pair sr = mad(two, s1, mul(splat(-1.0f), s23));
+    const T sq = mad(mtwo, syz, sxx);  // s_xy + s_xz - 2 s_yz
+    const T sr = mad(two, s1, mul(lit<T>(-1.0f), s23));
     m[5] = add(sr, sq);
-    const Pair d23 = sub(s2, s3), dxx = sub(sxy, sxz);
+    const T d23 = sub(s2, s3), dxx = sub(sxy, sxz);
     m[6] = add(d23, dxx);
     m[7] = sub(s7, s9);
     m[8] = sub(s15, s17);
@@ -216,14 +216,22 @@ __host__ __device__ __forceinline__ void philox4x32_10(uint32_t& x0, uint32_t& x
     }
 }
 
-__host__ __device__ __forceinline__ float uniform_open(uint32_t x)
+// The upper 23 bits of a word as the fraction of a float in [1, 2), by one
+// funnel shift: 0x7f above the word puts the exponent of 1 in front.
+__host__ __device__ __forceinline__ float one_to_two(uint32_t w)
 {
 #ifdef __CUDA_ARCH__
-    return __fmaf_rn((float)(x >> 9), 1.0f / 8388608.0f, 0.5f / 8388608.0f);
+    return __uint_as_float(__funnelshift_r(w, 0x7fu, 9));
 #else
-    return std::fmaf((float)(x >> 9), 1.0f / 8388608.0f, 0.5f / 8388608.0f);
+    const uint32_t u = (0x7fu << 23) | (w >> 9);
+    float f;
+    memcpy(&f, &u, sizeof(f));
+    return f;
 #endif
 }
+// ((w >> 9) + 1/2) 2^-23, in (0, 1), exact: the fraction minus 1 - 2^-24.
+constexpr float kHalfBelowOne = 0.999999940395355224609375f;
+__host__ __device__ __forceinline__ float uniform_open(uint32_t w) { return one_to_two(w) - kHalfBelowOne; }
 
 // ---------------------------------------------------------------------------
 // Launch-invariant parameters (kernel argument, by value).

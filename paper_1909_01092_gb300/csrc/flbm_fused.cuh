@@ -206,8 +206,8 @@ struct DensitySink {
         // where no node and no ring position gathers it.
         if (leaves(i)) xch[2 * (xch_slot(i) * size + pos) + l] = v;
     }
-    // Both components: one 8-byte store.
-    __device__ __forceinline__ void put(int i, Pair v, bool bounced)
+    // Both components, as the kernel has them: one 8-byte store.
+    __host__ __device__ __forceinline__ void put(int i, Pair v, bool bounced)
     {
         put_own(0, i, v.x, bounced);
         put_own(1, i, v.y, bounced);

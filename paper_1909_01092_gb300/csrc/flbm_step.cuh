@@ -48,20 +48,13 @@ __host__ __device__ __forceinline__ void philox_rk(uint32_t& x0, uint32_t& x1, u
 // their inputs and results here (u1 >= 2^-24, |angle| >= 2^-22, -2 ln u1 of
 // about 2^-23 at least) lie far above the subnormal range, where both forms
 // agree, and they skip the rescaling of subnormal inputs.
-// A word's upper 23 bits become the fraction of a float in [1, 2) by one
-// funnel shift (0x7f above the word puts the exponent of 1 in front), so the
-// uniforms need no integer conversion, which shares the slow pipe of the four
-// approximations: u = ((w >> 9) + 1/2) 2^-23 = float - (1 - 2^-24), exact.
-// The rest of the arithmetic is packed over the two pairs.
-__device__ __forceinline__ Pair one_to_two(uint32_t w1, uint32_t w3)
-{
-    return Pair{__uint_as_float(__funnelshift_r(w1, 0x7fu, 9)), __uint_as_float(__funnelshift_r(w3, 0x7fu, 9))};
-}
-
+// The uniforms (one_to_two, as uniform_open) need no integer conversion, which
+// shares the slow pipe of the four approximations. The rest of the arithmetic
+// is packed over the two pairs.
 __device__ __forceinline__ void box_muller2(uint32_t w1, uint32_t w2, uint32_t w3, uint32_t w4, float& za0, float& za1,
                                             float& zb0, float& zb1)
 {
-    const Pair u1 = add(one_to_two(w1, w3), splat(-0.999999940395355224609375f));
+    const Pair u1 = add(Pair{one_to_two(w1), one_to_two(w3)}, splat(-kHalfBelowOne));
     Pair lg, rs, s, c;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg.x) : "f"(u1.x));
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg.y) : "f"(u1.y));
@@ -72,7 +65,7 @@ __device__ __forceinline__ void box_muller2(uint32_t w1, uint32_t w2, uint32_t w
     // 2 pi (u2 - 1/2) with u2 = ((w2 >> 9) + 1/2) 2^-23.
     constexpr float kA = (float)6.283185307179586;
     constexpr float kB = (float)(6.283185307179586 * (0.5 / 8388608.0 - 0.5));
-    const Pair ang = mad(add(one_to_two(w2, w4), splat(-1.0f)), splat(kA), splat(kB));
+    const Pair ang = mad(add(Pair{one_to_two(w2), one_to_two(w4)}, splat(-1.0f)), splat(kA), splat(kB));
     asm("sin.approx.ftz.f32 %0, %1;" : "=f"(s.x) : "f"(ang.x));
     asm("cos.approx.ftz.f32 %0, %1;" : "=f"(c.x) : "f"(ang.x));
     asm("sin.approx.ftz.f32 %0, %1;" : "=f"(s.y) : "f"(ang.y));
@@ -115,7 +108,7 @@ struct LinkSums {
 };
 
 // Densities and momenta of both components from their populations.
-__device__ __forceinline__ void moments(const Pair f[19], Pair& rho, Pair j[3])
+__host__ __device__ __forceinline__ void moments(const Pair f[19], Pair& rho, Pair j[3])
 {
     const Pair s1 = add(f[1], f[2]), s2 = add(f[3], f[4]), s3 = add(f[5], f[6]);
     const Pair s7 = add(f[7], f[8]), s9 = add(f[9], f[10]), s11 = add(f[11], f[12]);
@@ -199,25 +192,12 @@ struct PushFrame {
             }
         }
     }
-    // Target of (l, i) and whether a wall bounced it: both candidate
-    // indices, then a select (no branch).
-    __host__ __device__ __forceinline__ uint32_t target(uint32_t n, int l, int i, const KParams& P, bool& wall) const
-    {
-        const int cx = cxv(i), cy = cyv(i), cz = czv(i);
-        const uint32_t need_p = (cx > 0 ? 1u : 0u) | (cy > 0 ? 2u : 0u) | (cz > 0 ? 4u : 0u);
-        const uint32_t need_m = (cx < 0 ? 1u : 0u) | (cy < 0 ? 2u : 0u) | (cz < 0 ? 4u : 0u);
-        wall = ((wallp & need_p) | (wallm & need_m)) != 0u;
-        const uint32_t back_idx = n + P.dirN[19 * l + oppv(i)];
-        int off = 0;
-        if (cx) off += cx > 0 ? offp[0] : offm[0];
-        if (cy) off += cy > 0 ? offp[1] : offm[1];
-        if (cz) off += cz > 0 ? offp[2] : offm[2];
-        const uint32_t push_idx = n + (uint32_t)off + P.dirN[19 * l + i];
-        return wall ? back_idx : push_idx;
-    }
-    // The same target as a byte offset from the first slot of the pair of
-    // opposite directions i belongs to (directions 2 k - 1 and 2 k; the rest
-    // direction alone), the same for both components.
+    // First direction of the pair of opposite directions i belongs to
+    // (directions 2 k - 1 and 2 k; the rest direction alone).
+    static __host__ __device__ constexpr int pair_of(int i) { return i == 0 || (i & 1) ? i : i - 1; }
+    // Target of population i as a byte offset from slot pair_of(i) of either
+    // component, and whether a wall bounced it: both candidate offsets, then
+    // a select (no branch).
     __host__ __device__ __forceinline__ uint32_t target_bytes(uint32_t n, int i, const KParams& P, bool& wall) const
     {
         const int cx = cxv(i), cy = cyv(i), cz = czv(i);
@@ -229,10 +209,15 @@ struct PushFrame {
         if (cx) off += cx > 0 ? offp[0] : offm[0];
         if (cy) off += cy > 0 ? offp[1] : offm[1];
         if (cz) off += cz > 0 ? offp[2] : offm[2];
-        const bool second = i != 0 && i % 2 == 0;
+        const bool second = pair_of(i) != i;
         const uint32_t push = n + (uint32_t)off + (second ? N : 0u);
         const uint32_t back = n + (i != 0 && !second ? N : 0u);
         return 4u * (wall ? back : push);
+    }
+    // The same target as an index into the populations of component l.
+    __host__ __device__ __forceinline__ uint32_t target(uint32_t n, int l, int i, const KParams& P, bool& wall) const
+    {
+        return P.dirN[19 * l + pair_of(i)] + target_bytes(n, i, P, wall) / 4u;
     }
 };
 
@@ -248,7 +233,7 @@ struct NoSink {
 
 // sqrt(1 / b_k): the noise amplitude of normalised mode k >= 4 per
 // sqrt(3 kT rho_l) when its relaxation time is 1.
-__device__ constexpr float noise_unit(int k)
+__host__ __device__ constexpr float noise_unit(int k)
 {
     return k == 4 ? 1.22474487139158905f      // b = 2/3
            : k == 5 ? 0.866025403784438647f   // 4/3
@@ -342,7 +327,7 @@ __device__ __forceinline__ void load_modes(const In& in, const KParams& P, NodeS
 
 // Differences of opposite neighbours first: they are close in value.
 template <bool TAU1, class In>
-__device__ __forceinline__ void load_force(const In& in, NodeState<TAU1>& s)
+__host__ __device__ __forceinline__ void load_force(const In& in, NodeState<TAU1>& s)
 {
     const Pair d1 = sub(in.psi(1), in.psi(2)), d2 = sub(in.psi(3), in.psi(4)), d3 = sub(in.psi(5), in.psi(6));
     const Pair d7 = sub(in.psi(7), in.psi(8)), d9 = sub(in.psi(9), in.psi(10));
@@ -500,7 +485,7 @@ __device__ __forceinline__ void collide_push(int x, int y, int z, uint32_t n, co
         }
         bool wall;
         const uint32_t to = frame.target_bytes(n, i, P, wall);
-        const int pair = i == 0 ? 0 : (i & 1) ? i : i - 1;
+        const int pair = PushFrame::pair_of(i);
         *at(fout + P.dirN[pair], to) = fo[i].x;
         *at(fout + P.dirN[19 + pair], to) = fo[i].y;
         if constexpr (Sink::active) sink->put(i, fo[i], wall);
@@ -834,7 +819,7 @@ __device__ __forceinline__ double event_value(int k, const double r[3], const do
 // times 4 (R + 4) and a few ulps), else in FP64: few nodes need the slow pipe.
 struct SphereTest {
     float x[3], R2, margin;
-    __device__ __forceinline__ SphereTest(const double X[3], const KParams& P)
+    __host__ __device__ __forceinline__ SphereTest(const double X[3], const KParams& P)
     {
         const float R = (float)P.R;
 #pragma unroll
@@ -842,7 +827,7 @@ struct SphereTest {
         R2 = R * R;
         margin = 1e-6f * ((R + 4.0f) * (float)max(P.lx, max(P.ly, P.lz)) + 8.0f * R2) + 1e-5f;
     }
-    __device__ __forceinline__ bool inside(const int c[3], const double X[3], const KParams& P) const
+    __host__ __device__ __forceinline__ bool inside(const int c[3], const double X[3], const KParams& P) const
     {
         const int L[3] = {P.lx, P.ly, P.lz};
         float s = 0.0f;
