@@ -510,7 +510,6 @@ int flbm_create(const flbm_params* p, void* f_dev, size_t f_dev_bytes, void* str
         cudaMalloc(&h->box_counts, sizeof(int) * h->box_blocks) != cudaSuccess ||
         cudaMalloc(&h->box_parts, sizeof(double) * 8 * h->box_blocks) != cudaSuccess ||
         cudaMalloc(&h->obs_parts, sizeof(double) * kObsValues * obs_geom(k).blocks) != cudaSuccess ||
-        cudaMalloc(&h->obs_marked, sizeof(int) * obs_geom(k).blocks) != cudaSuccess ||
         cudaMalloc(&h->obs_out, sizeof(ObsOut)) != cudaSuccess)
         return bail(FLBM_E_NOMEM);
 
@@ -736,7 +735,7 @@ int flbm_observables(flbm_t* h, flbm_obs* out)
 {
     if (!h || !out) return fail(h, FLBM_E_INVAL, "NULL argument");
     const KParams& k = h->kp;
-    CK(h, launch_observe(h->fbuf[h->cur], h->st, h->masks, h->obs_parts, h->obs_marked, h->obs_out, k, h->stream));
+    CK(h, launch_observe(h->fbuf[h->cur], h->st, h->masks, h->obs_parts, h->obs_out, k, h->stream));
     ObsOut r;
     CK(h, cudaMemcpyAsync(&r, h->obs_out, sizeof(r), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
@@ -902,7 +901,6 @@ void flbm_destroy(flbm_t* h)
     cudaFree(h->box_counts);
     cudaFree(h->box_parts);
     cudaFree(h->obs_parts);
-    cudaFree(h->obs_marked);
     cudaFree(h->obs_out);
     cudaFree(h->scratch_rho);
     cudaFree(h->traj_dev);

@@ -238,7 +238,6 @@ struct flbm_ens {
     };
     std::vector<RepLaunch> rep_launches[4];
     double* obs_parts = nullptr;   // for the replica with the most blocks of k_obs
-    int* obs_marked = nullptr;
     ObsOut* obs_out = nullptr;
     long long obs_blocks = 0;
     int cur = 0;                   // all replicas read f[cur] in the next step
@@ -430,7 +429,6 @@ int allocate(flbm_ens* e)
     ECK(e, cudaMemsetAsync(e->arena, 0, off, e->stream));
     if (cudaMalloc(&e->d_reps, sizeof(RepDesc) * e->n) != cudaSuccess ||
         cudaMalloc(&e->obs_parts, sizeof(double) * kObsValues * e->obs_blocks) != cudaSuccess ||
-        cudaMalloc(&e->obs_marked, sizeof(int) * e->obs_blocks) != cudaSuccess ||
         cudaMalloc(&e->obs_out, sizeof(ObsOut)) != cudaSuccess)
         return efail(e, FLBM_E_NOMEM, "ensemble descriptors");
     char* base = static_cast<char*>(e->arena);
@@ -718,7 +716,7 @@ int flbm_ensemble_observables(flbm_ens_t* e, int32_t r, flbm_obs* out)
     if (!e || !out || r < 0 || r >= e->n) return efail(e, FLBM_E_INVAL, "invalid argument");
     const KParams& k = e->kp[r];
     const RepDesc& d = e->rd[r];
-    ECK(e, launch_observe(d.f[e->cur], d.st, d.masks, e->obs_parts, e->obs_marked, e->obs_out, k, e->stream));
+    ECK(e, launch_observe(d.f[e->cur], d.st, d.masks, e->obs_parts, e->obs_out, k, e->stream));
     ObsOut res;
     ECK(e, cudaMemcpyAsync(&res, e->obs_out, sizeof(res), cudaMemcpyDeviceToHost, e->stream));
     ECK(e, cudaStreamSynchronize(e->stream));
@@ -749,7 +747,6 @@ void flbm_ensemble_destroy(flbm_ens_t* e)
     cudaFree(e->d_reps);
     cudaFree(e->d_items);
     cudaFree(e->obs_parts);
-    cudaFree(e->obs_marked);
     cudaFree(e->obs_out);
     delete e;
 }

@@ -44,7 +44,6 @@ struct flbm_sim {
     int box_blocks = 0;
     long long ncand = 0;
     double* obs_parts = nullptr;   // per block of k_obs: its sums, value by value
-    int* obs_marked = nullptr;     // per block of k_obs: redo in FP64
     flbm::ObsOut* obs_out = nullptr;
     float* scratch_rho = nullptr;
     DevState* traj_dev = nullptr;  // per-step particle records of flbm_run_host
