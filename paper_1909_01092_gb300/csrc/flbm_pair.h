@@ -53,6 +53,14 @@ __host__ __device__ __forceinline__ Pair mad(Pair a, Pair b, Pair c)
 // a - b: the product with -1 is exact
 __host__ __device__ __forceinline__ Pair sub(Pair a, Pair b) { return mad(b, splat(-1.0f), a); }
 
+// s + e = a + b exactly, s = fl(a + b) (Knuth's two-sum)
+__host__ __device__ __forceinline__ void two_sum(Pair a, Pair b, Pair& s, Pair& e)
+{
+    s = add(a, b);
+    const Pair bb = sub(s, a);
+    e = add(sub(a, sub(s, bb)), sub(b, bb));
+}
+
 __host__ __device__ __forceinline__ float add(float a, float b) { return a + b; }
 __host__ __device__ __forceinline__ float sub(float a, float b) { return a - b; }
 __host__ __device__ __forceinline__ float mul(float a, float b) { return a * b; }

@@ -9,6 +9,8 @@
 //  6. SphereTest decides as node_inside does, for nodes at distance
 //     R (1 + e), e from 1e-16 to 1, on axes of 8 to 2^20 nodes, across
 //     periodic wraps and beside walls, with most nodes decided in float.
+//  7. pop_sums: populations of sizes 2^-30 to 1, either sign, to 19 roundings of
+//     FP64 of their magnitudes.
 // Prints one line and returns 0 when all hold.
 #include <cmath>
 #include <cstdio>
@@ -141,6 +143,22 @@ int main()
         ++nodes;
         inside += want;
         in_float += std::fabs(e) * 2.0 * P.R * P.R > 2.0 * s.margin;
+    }
+    // 7.
+    for (int t = 0; t < 20000; ++t) {
+        const long long N = 1 + (long long)(g() % 5), m = (long long)(g() % (unsigned long long)N);
+        std::vector<float> f((size_t)(38 * N));
+        for (float& v : f) v = (float)((g() % 2 ? 1.0 : -1.0) * std::exp2(-30.0 * unit(g)));
+        double got[2];
+        pop_sums(f.data(), m, N, got);
+        for (int l = 0; l < 2; ++l) {
+            long double sum = 0.0L, size = 0.0L;
+            for (int i = 0; i < 19; ++i) {
+                sum += f[(19 * l + i) * N + m];
+                size += std::fabs(f[(19 * l + i) * N + m]);
+            }
+            failed += std::fabs((double)(got[l] - sum)) > (double)(19.0L * size) * 0x1p-53;
+        }
     }
     failed += !(nodes > 100000 && inside > nodes / 4 && in_float > nodes / 20);
     std::printf("nodes %lld inside %lld clear %lld failed %d\n", nodes, inside, in_float, failed);
