@@ -75,10 +75,13 @@ __device__ __forceinline__ void box_muller2(uint32_t w1, uint32_t w2, uint32_t w
     zb1 = -r.y * s.y;
 }
 
-// 1 / x and sqrt(x) for finite x > 0 (sqrt: x >= 0) from the hardware's
-// approximations and one Newton step each, to within an ulp, without the
-// branches and calls of the general routines. Zero gives 0 for the square
-// root; a NaN stays one.
+// 1 / x and sqrt(x) from the hardware's approximations and one Newton step
+// each, without the branches and calls of the general routines (__frcp_rn and
+// __fsqrt_rn: 5544 -> 5715 us for 8 steps of 128x128x512 with noise). Within
+// half an ulp and 2^-18 of one for 2^-126 <= x <= 2^126 and 2^-100 <= x, where
+// a sweep of mantissas and exponents found CUDA's correctly rounded results
+// every time; a smaller root is within 4 ulp, as its residual runs out of
+// exponents. The root of zero is zero; a NaN stays one.
 __device__ __forceinline__ float recip_newton(float x)
 {
     float r;
@@ -88,7 +91,7 @@ __device__ __forceinline__ float recip_newton(float x)
 __device__ __forceinline__ float sqrt_newton(float x)
 {
     float y;
-    asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(x, 1.17549435e-38f)));
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(x, 1.401298464e-45f)));  // the least float: a finite y for zero
     const float s = __fmul_rn(x, y);
     return __fmaf_rn(__fmaf_rn(-s, s, x), __fmul_rn(0.5f, y), s);
 }
