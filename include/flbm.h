@@ -417,11 +417,10 @@ typedef struct flbm_ens_config {
                             1 interleaved (item k of every replica, then item k+1),
                             2 replica after replica, largest lattice first */
     int32_t ctas_per_sm; /* persistent blocks per SM of every batched launch (1..8);
-                            0: one block per work item. The bulk collide runs in
-                            launches of up to 48 replicas of similar tile counts
-                            whose descriptors are a kernel parameter, one block
-                            per tile, unless ctas_per_sm > 0 and that takes more
-                            than four launches a step */
+                            0: one block per work item. The bulk collide takes the
+                            descriptors of up to 48 replicas a launch as a kernel
+                            parameter; an SM holds at most four of its blocks (256
+                            threads), so from 4 on it runs one block per item */
     int32_t tile_policy; /* 0: tile width min(32, next power of two >= lx), as flbm_create;
                             1: the largest of 32, 16, 8 that divides lx (else as 0) */
 } flbm_ens_config;

@@ -10,8 +10,8 @@
 // pointers) in shared memory and runs the same device bodies as the
 // single-simulation kernels, so each replica computes exactly what
 // flbm_create/flbm_step would. The bulk collide instead takes the descriptors
-// of up to kChunkReps replicas as a kernel parameter (kb_bulk_rep), unless that
-// takes many launches a step in a persistent configuration. The step sequence (densities; density shell;
+// of up to kChunkReps replicas as a kernel parameter: kept in shared memory
+// they cost the update its registers. The step sequence (densities; density shell;
 // collide-stream of the bulk tiles; on a side stream meanwhile the virtual
 // layer and the near tiles, whose launch ends with each replica's particle
 // update; next-position masks and cover/uncover ending with each replica's
@@ -91,8 +91,9 @@ __device__ __forceinline__ TileCoord tile_of(const Item& it, const KParams& P)
         const KParams& P = sR.P;
 #define FLBM_END_ITEMS }
 
-// Persistent blocks (PERSIST) keep a node's 38 loads in flight, in 64
-// registers: there are only a few of them. One block per item does better with
+// Persistent blocks (PERSIST) load a node's 38 populations before they add them
+// up, in 64 registers and 192 bytes of spills a thread: there are only a few
+// of them to hide a load behind another block's. One block per item does better with
 // 32 registers and eight blocks per SM, among which the descriptors' staging
 // hides (128 replicas: 1.04 ms a step against 1.19 ms).
 template <bool PERSIST>
@@ -115,18 +116,6 @@ static __global__ void __launch_bounds__(256) kb_shell(const RepDesc* __restrict
         shell_node(it.y * 256LL + threadIdx.x, sR.psi, sR.st, sR.masks, P);
     else
         virtual_node((it.y - nbs) * 256 + threadIdx.x, sR.psi, sR.st, sR.masks, P);
-    FLBM_END_ITEMS
-}
-
-// Two blocks per SM: the descriptor read from shared memory leaves the update
-// 216 bytes of spills at three.
-template <bool NOISE, bool TAU1>
-static __global__ void __launch_bounds__(256, 2)
-    kb_bulk(const RepDesc* __restrict__ reps, const Item* __restrict__ items, int nitems, int par)
-{
-    FLBM_FOR_ITEMS
-    const TileCoord c = tile_of(it, P);
-    bulk_tile<NOISE, TAU1>(c.bx, c.by, c.bz, c.tx, c.ty, sR.f[par], sR.f[1 - par], sR.psi, sR.st, P);
     FLBM_END_ITEMS
 }
 
@@ -159,8 +148,36 @@ static __global__ void __launch_bounds__(kBulkThreads<NOISE>, kBulkBlocks<NOISE>
     bulk_tile<NOISE, TAU1>(bx, by, bz, tx, ty, R.f[par], R.f[1 - par], R.psi, R.st, P);
 }
 
-// Two blocks per SM, without spills (step of the confinement channels, where
-// most tiles are near: 1.13 ms against 1.32 ms at three, bulk lists included).
+// The bulk collide over a work list (packing, ctas_per_sm), its descriptors the
+// same kernel parameter: item x counts within the chunk, kBulkParts blocks
+// share an item. Without LOOP a block does one item; with it, persistent blocks
+// stay within the caller's ctas_per_sm, two per SM: three would leave the
+// update 80 registers and 24 to 184 bytes of spills. A step of 128 replicas
+// with ctas_per_sm 1 / 2 / 3 / 4 takes 2.10 / 1.51 / 1.41 / 1.12 ms, of 15
+// channels of 60x60x120 1.61 / 1.22 / 1.13 / 0.91 ms, against 2.64 / 2.03 /
+// 1.72 / 1.64 and 2.06 / 1.56 / 1.31 / 1.25 ms with persistent blocks that read
+// their descriptors from shared memory and an update without packed arithmetic.
+constexpr int kLoopBlocks = 2;
+template <bool NOISE, bool TAU1, bool LOOP>
+static __global__ void __launch_bounds__(kBulkThreads<NOISE>, LOOP ? kLoopBlocks * kBulkParts<NOISE> : kBulkBlocks<NOISE>)
+    kb_bulk(const __grid_constant__ RepChunk c, const Item* __restrict__ items, int nitems, int par)
+{
+    constexpr int parts = kBulkParts<NOISE>;
+    int i = blockIdx.x / parts;
+    do {
+        const Item it = items[i];
+        const RepDesc& R = c.r[it.x];
+        const KParams& P = R.P;
+        const int tid = threadIdx.x + kBulkThreads<NOISE> * (blockIdx.x % parts);
+        const int tx = tid & (P.tx - 1), ty = tid >> (__ffs(P.tx) - 1);
+        bulk_tile<NOISE, TAU1>(it.y, it.z, it.w, tx, ty, R.f[par], R.f[1 - par], R.psi, R.st, P);
+        i += gridDim.x / parts;
+    } while (LOOP && i < nitems);
+}
+
+// Two blocks per SM: 16 bytes of spills a thread with noise, 244 with noise and
+// relaxation times that are not 1, none else (step of the confinement channels,
+// where most tiles are near: 1.13 ms against 1.32 ms at three).
 template <bool NOISE, bool TAU1>
 static __global__ void __launch_bounds__(256, 2)
     kb_near(const RepDesc* __restrict__ reps, const Item* __restrict__ items, int nitems, int par)
@@ -227,14 +244,15 @@ struct flbm_ens {
     Item* d_items = nullptr;
     size_t items_cap = 0;
     long long off[W_COUNT + 1] = {};  // work list k = d_items[off[k] .. off[k+1])
-    // Bulk collide launches of one block per tile, per variant: replicas of
-    // similar tile counts grouped, kChunkReps at most per launch; in use with
-    // ctas_per_sm 0, and otherwise while they are few.
-    bool bulk_by_reps = false;
+    // Bulk collide launches, per variant, kChunkReps replicas at most each.
+    // ctas_per_sm 0: a block per tile, replicas of similar tile counts
+    // grouped. Otherwise nitems work items of d_items from off.
     struct RepLaunch {
         RepChunk c;
         int n = 0;
         int max_blocks = 0;
+        long long off = 0;
+        int nitems = 0;
     };
     std::vector<RepLaunch> rep_launches[4];
     double* obs_parts = nullptr;   // for the replica with the most blocks of k_obs
@@ -317,44 +335,61 @@ int apply_config(flbm_ens* e)
         if (w == W_VIRT) return make_int4(r, (int)(blocks_of(k, W_SHELL) + b), 0, 0);
         return make_int4(r, (int)b, 0, 0);
     };
+    // Appends the blocks of the replicas in list w in the order of the packing;
+    // label gives an item's x.
+    auto append = [&](const std::vector<int>& reps, int w, auto label) {
+        long long most = 0;
+        if (e->cfg.packing == 1)
+            for (int r : reps) most = std::max(most, blocks_of(e->kp[r], w));
+        auto push = [&](size_t at, long long b) {
+            Item it = item(reps[at], b, w);
+            it.x = label(at);
+            items.push_back(it);
+        };
+        for (long long b = 0; b < most; ++b)
+            for (size_t at = 0; at < reps.size(); ++at)
+                if (b < blocks_of(e->kp[reps[at]], w)) push(at, b);
+        if (e->cfg.packing != 1)
+            for (size_t at = 0; at < reps.size(); ++at)
+                for (long long b = 0, nb = blocks_of(e->kp[reps[at]], w); b < nb; ++b) push(at, b);
+    };
     for (int w = 0; w < W_COUNT; ++w) {
         e->off[w] = (long long)items.size();
-        if (e->cfg.packing == 1) {
-            long long most = 0;
-            for (int r = 0; r < e->n; ++r) most = std::max(most, blocks_of(e->kp[r], w));
-            for (long long b = 0; b < most; ++b)
-                for (int r = 0; r < e->n; ++r)
-                    if (b < blocks_of(e->kp[r], w)) items.push_back(item(r, b, w));
-        } else {
-            for (int r : order)
-                for (long long b = 0, nb = blocks_of(e->kp[r], w); b < nb; ++b) items.push_back(item(r, b, w));
-        }
+        if (w < W_BULK || w >= W_BULK + 4) append(order, w, [&](size_t at) { return order[at]; });
     }
     e->off[W_COUNT] = (long long)items.size();
-    // Bulk launches with descriptor chunks, per variant (group_by_blocks;
-    // the blocks past a replica's own tiles return at once).
+    // Bulk launches. A block per tile: groups of similar sizes (group_by_blocks;
+    // the blocks past a replica's own tiles return at once). Work lists: the
+    // replicas as the packing orders them.
     for (int k = 0; k < 4; ++k) {
         std::vector<long long> tiles(e->n);
         for (int r = 0; r < e->n; ++r) {
             tiles[r] = blocks_of(e->kp[r], W_BULK + k);
             if (tiles[r] > 0x7fffffffLL) return efail(e, FLBM_E_INVAL, "too many tiles in one replica");
         }
+        std::vector<std::vector<int>> groups;
+        if (e->cfg.ctas_per_sm == 0) {
+            groups = group_by_blocks(tiles, kChunkReps);
+        } else {
+            for (int r : order) {
+                if (tiles[r] == 0) continue;
+                if (groups.empty() || groups.back().size() == kChunkReps) groups.emplace_back();
+                groups.back().push_back(r);
+            }
+        }
         auto& ch = e->rep_launches[k];
         ch.clear();
-        for (const auto& g : group_by_blocks(tiles, kChunkReps)) {
+        for (const auto& g : groups) {
             ch.emplace_back();
-            ch.back().max_blocks = (int)tiles[g[0]];
-            for (int r : g) ch.back().c.r[ch.back().n++] = e->rd[r];
+            auto& l = ch.back();
+            l.max_blocks = (int)tiles[g[0]];
+            for (int r : g) l.c.r[l.n++] = e->rd[r];
+            if (e->cfg.ctas_per_sm == 0) continue;
+            l.off = (long long)items.size();
+            append(g, W_BULK + k, [](size_t at) { return (int)at; });
+            l.nitems = (int)((long long)items.size() - l.off);
         }
     }
-    // The descriptors in the constant bank instead of shared memory leave the
-    // update its registers: 15 channels of 60x60x120 take 480 us a step through
-    // the lists' kernel; their step falls from 1.06 to 0.91 ms with these. Persistent
-    // configurations keep the lists only where the replicas' sizes would ask
-    // for many launches.
-    size_t reps = 0;
-    for (int k = 0; k < 4; ++k) reps += e->rep_launches[k].size();
-    e->bulk_by_reps = e->cfg.ctas_per_sm == 0 || reps <= 4;
     if (items.size() > (size_t)0x7fffffff) return efail(e, FLBM_E_INVAL, "too many work items");
     if (items.size() > e->items_cap) {
         cudaFree(e->d_items);
@@ -474,17 +509,37 @@ int launch_list(flbm_ens* e, int w, void (*kern)(const RepDesc*, const Item*, in
     return launch_on(e, e->stream, w, kern, what, args...);
 }
 
-// The bulk collide launches with descriptor chunks.
-int launch_bulk_reps(flbm_ens* e, int par)
+template <bool LOOP>
+void launch_bulk_list(int variant, unsigned blocks, unsigned threads, cudaStream_t s, const RepChunk& c,
+                      const Item* items, int nitems, int par)
 {
-    void (*kern[4])(const RepChunk, int) = {kb_bulk_rep<false, false>, kb_bulk_rep<false, true>,
+    void (*kern[4])(const RepChunk, const Item*, int, int) = {kb_bulk<false, false, LOOP>, kb_bulk<false, true, LOOP>,
+                                                              kb_bulk<true, false, LOOP>, kb_bulk<true, true, LOOP>};
+    kern[variant]<<<blocks, threads, 0, s>>>(c, items, nitems, par);
+}
+
+// The bulk collide launches: a block per tile, or over the lists within the
+// caller's bound. An SM holds kBulkBlocks<false> = 4 blocks of 256 threads of a
+// launch that does not loop, seven half ones with noise, which is as much.
+int launch_bulk(flbm_ens* e, int par)
+{
+    void (*tile[4])(const RepChunk, int) = {kb_bulk_rep<false, false>, kb_bulk_rep<false, true>,
                                             kb_bulk_rep<true, false>, kb_bulk_rep<true, true>};
+    const int ctas = e->cfg.ctas_per_sm;
     for (int k = 0; k < 4; ++k)
-        for (const auto& ch : e->rep_launches[k]) {
+        for (const auto& l : e->rep_launches[k]) {
             const unsigned parts = k >= 2 ? kBulkParts<true> : kBulkParts<false>;
             const unsigned threads = k >= 2 ? kBulkThreads<true> : kBulkThreads<false>;
-            kern[k]<<<dim3(parts * (unsigned)ch.max_blocks, (unsigned)ch.n), threads, 0, e->stream>>>(ch.c, par);
-            if (int rc = elaunch(e, "kb_bulk_rep")) return rc;
+            const unsigned blocks =
+                parts * (unsigned)bulk_list_blocks(l.nitems, ctas, kBulkBlocks<false>, kLoopBlocks, e->nsm);
+            const Item* items = e->d_items + l.off;
+            if (ctas == 0)
+                tile[k]<<<dim3(parts * (unsigned)l.max_blocks, (unsigned)l.n), threads, 0, e->stream>>>(l.c, par);
+            else if (ctas >= kBulkBlocks<false>)
+                launch_bulk_list<false>(k, blocks, threads, e->stream, l.c, items, l.nitems, par);
+            else
+                launch_bulk_list<true>(k, blocks, threads, e->stream, l.c, items, l.nitems, par);
+            if (int rc = elaunch(e, "kb_bulk")) return rc;
         }
     return FLBM_OK;
 }
@@ -518,14 +573,7 @@ int ens_step(flbm_ens* e)
         if (int rc = launch_on(e, e->side, W_NEAR + 3, kb_near<true, true>, "kb_near", par)) return rc;
         ECK(e, cudaEventRecord(e->join_ev, e->side));
     }
-    if (e->bulk_by_reps) {
-        if (int rc = launch_bulk_reps(e, par)) return rc;
-    } else {
-        if (int rc = launch_list(e, W_BULK + 0, kb_bulk<false, false>, "kb_bulk", par)) return rc;
-        if (int rc = launch_list(e, W_BULK + 1, kb_bulk<false, true>, "kb_bulk", par)) return rc;
-        if (int rc = launch_list(e, W_BULK + 2, kb_bulk<true, false>, "kb_bulk", par)) return rc;
-        if (int rc = launch_list(e, W_BULK + 3, kb_bulk<true, true>, "kb_bulk", par)) return rc;
-    }
+    if (int rc = launch_bulk(e, par)) return rc;
     if (near) ECK(e, cudaStreamWaitEvent(e->stream, e->join_ev, 0));
     if (int rc = launch_list(e, W_COVER, kb_cover, "kb_cover", par)) return rc;
     if (int rc = launch_list(e, W_FINISH, kb_finish, "kb_finish")) return rc;

@@ -149,6 +149,16 @@ inline std::vector<std::vector<int>> group_by_blocks(const std::vector<long long
     return groups;
 }
 
+// Items that the blocks of a bulk launch over a list of nitems start with: all
+// of them, a block each, where the caller's bound of ctas blocks per SM is no
+// lower than the `resident` an SM holds of the launch anyway (it then evens
+// itself out over the SMs); else as many as persistent blocks stay within the
+// bound, of which an SM holds `loop`.
+inline int bulk_list_blocks(int nitems, int ctas, int resident, int loop, int nsm)
+{
+    return ctas >= resident ? nitems : std::min(nitems, std::min(ctas, loop) * nsm);
+}
+
 // Particle record at creation (Section 3, Eq. (fp)): sphere of radius R at
 // pos0, at rest, mass 4/3 pi R^3 rho_p, moment of inertia 2/5 m_p R^2.
 inline DevState initial_state(const flbm_params& p, const KParams& k)
