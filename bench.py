@@ -41,10 +41,10 @@ FALLBACK_HBM_GBS = 6800.0
 # 128x128x512 channel, from an ncu capture of one bulk-kernel launch on the
 # 128x128x128 channel (populations larger than L2), scaled by bulk nodes:
 # B per bulk node x 8,331,264 bulk nodes + 9.9 MB by the near launch.
-COLLIDE_TRAFFIC_PER_BULK_NODE = 287.7
+COLLIDE_TRAFFIC_PER_BULK_NODE = 287.8
 COLLIDE_TRAFFIC_BYTES = COLLIDE_TRAFFIC_PER_BULK_NODE * 8331264 + 9.9e6
 # Thread instructions per node of the noisy bulk collide kernel (same capture).
-COLLIDE_INST_PER_NODE = 1368.1
+COLLIDE_INST_PER_NODE = 1371.1
 SMS, SCHEDULERS_PER_SM = 152, 4
 
 

@@ -112,8 +112,8 @@ __host__ __device__ __forceinline__ void to_modes(const T f[19], T m[19])
 // by which a step's mass grew, two thirds. (1/18 and 1/36 are 2^-27 too large,
 // f_i 1e-8; correcting all nine of their products would take another 0.5 to 1 %
 // of a step.) Populations of the paper's mixture after 8 steps are 0.8e-7 off
-// FP64, 1.6e-7 with the float alone; 8 steps of 128x128x512 with noise take 5590
-// us, 5560 with the float alone.
+// FP64, 1.6e-7 with the float alone; 8 steps of 128x128x512 with noise take 5565
+// us, 5550 with the float alone.
 constexpr float kThirdLow = -9.934107481e-9f;
 
 // Back transform f_i = w_i sum_k e_k(c_i) n_k with n_k = m_k / b_k already
